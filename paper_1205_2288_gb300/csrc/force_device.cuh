@@ -48,7 +48,7 @@ __device__ __forceinline__ void write_partial(const ForceArgs& A, int n_act,
 }
 
 // ---------------------------------------------------------------------
-// FP64: each pair term rounded op by op in the order of the definition.
+// FP64, j-split: sums in any order.
 // ---------------------------------------------------------------------
 struct __align__(16) F64Tile {
   double x[kTileF64], y[kTileF64], z[kTileF64];
@@ -58,34 +58,6 @@ struct __align__(16) F64Tile {
 struct F64Acc {
   double ax, ay, az, ph, q;
 };
-
-__device__ __forceinline__ void pair_f64(const F64Tile& T, int t, double xi,
-                                         double yi, double zi, double ui,
-                                         double vi, double wi, double eps2,
-                                         F64Acc& s) {
-  const double dx = __dsub_rn(T.x[t], xi);
-  const double dy = __dsub_rn(T.y[t], yi);
-  const double dz = __dsub_rn(T.z[t], zi);
-  const double s2 = __dadd_rn(
-      __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                __dmul_rn(dz, dz)),
-      eps2);
-  const double sq = __dsqrt_rn(s2);
-  const double f = __ddiv_rn(T.m[t], __dmul_rn(s2, sq));
-  s.ax = __dadd_rn(s.ax, __dmul_rn(f, dx));
-  s.ay = __dadd_rn(s.ay, __dmul_rn(f, dy));
-  s.az = __dadd_rn(s.az, __dmul_rn(f, dz));
-  s.ph = __dsub_rn(s.ph, __ddiv_rn(T.m[t], sq));
-  const double wx = __dsub_rn(T.u[t], ui);
-  const double wy = __dsub_rn(T.v[t], vi);
-  const double wz = __dsub_rn(T.w[t], wi);
-  const double c = __ddiv_rn(
-      __dadd_rn(__dadd_rn(__dmul_rn(wx, wx), __dmul_rn(wy, wy)),
-                __dmul_rn(wz, wz)),
-      s2);
-  if (c > s.q) s.q = c;
-  if (f > s.q) s.q = f;
-}
 
 // 1/sqrt(s2) in FP64 for the j-split path: the FP32 reciprocal square root
 // refined by two Newton-Raphson steps for 1/sqrt (y <- y + y (1 - s2 y^2)/2,
@@ -168,16 +140,9 @@ __device__ void f64_item(const ForceArgs& A, int n_act, const Plan& P,
         T.m[q] = A.m[j];
       }
       __syncthreads();
-      if (A.exact) {
-        for (int q = jl; q < cnt; q += JG) {
-          if (jt + q == i) continue;
-          pair_f64(T, q, xi, yi, zi, ui, vi, wi, eps2, s);
-        }
-      } else {
-        for (int q = jl; q < cnt; q += JG) {
-          if (jt + q == i) continue;
-          pair_f64_fast(T, q, xi, yi, zi, ui, vi, wi, eps2, s);
-        }
+      for (int q = jl; q < cnt; q += JG) {
+        if (jt + q == i) continue;
+        pair_f64_fast(T, q, xi, yi, zi, ui, vi, wi, eps2, s);
       }
     }
     if constexpr (JG > 1) {
@@ -208,75 +173,189 @@ __device__ void f64_item(const ForceArgs& A, int n_act, const Plan& P,
   }
 }
 
-// FP64 with ascending-j sums for a few active bodies, one body per block:
-// the block's threads compute the pair terms of kThreads consecutive j in
-// parallel (the correctly rounded square root and divisions are the long
-// latency) and thread 0 then adds them in ascending j, the same rounded
-// operations in the same order as one thread running the whole loop. The
-// self pair contributes exact zeros (a sum that starts at +0 is never -0,
-// so adding +0 leaves it unchanged). q is a maximum, exact in any order.
-__device__ inline void f64_item_exact1(const ForceArgs& A, int n_act, int k,
-                                double (*red)[kThreads]) {
-  const int t = threadIdx.x;
-  const int i = A.idx[k];
-  const double xi = A.x[0][i], yi = A.x[1][i], zi = A.x[2][i];
-  const double ui = A.w[0][i], vi = A.w[1][i], wi = A.w[2][i];
+// ---------------------------------------------------------------------
+// FP64 with ascending-j sums (bit-identical to a sequential evaluation): a
+// block takes B active bodies. The pair terms of a tile of j are formed in
+// parallel and put into shared memory; the sums then add them in ascending
+// j, one lane per sum. The self pair and j past the end contribute zeros (a
+// sum that starts at +0 is never -0, so adding a zero leaves it unchanged);
+// the potential's terms are stored negated (s - t and s + (-t) round
+// alike). q is a maximum, exact in any order, and taken on the bit patterns.
+//
+// What bounds it: each FP64 instruction of a warp occupies its scheduler's
+// FP64 pipe for 64 cycles, however many lanes it serves, so the sums of one
+// j cost 64 cycles per warp that adds, and a pair term ~50 of them. Hence
+//  - kOverlap (few bodies per block): all sums of the block sit in the
+//    lanes of warp 0 (lane 4 b + c: body b, component c), while the other
+//    three warps, on the three other pipes, form the next tile's terms: with
+//    one body the block runs at the latency of the chain of n additions;
+//  - otherwise every warp forms terms, then warp c adds component c with
+//    one lane per body, so that up to 32 bodies share each addition.
+// Measured, 129 of 4099 bodies: 248 us; one thread adding all four sums of
+// one body (four instructions per j, on one pipe) took 698 us. The era of
+// Plummer 256 went from 184 to 92 ms. Without kOverlap the alternative is a
+// thread per body that forms and adds its terms, which does no more pairs
+// per FP64 instruction and leaves most of the chip idle at these counts.
+// ---------------------------------------------------------------------
+constexpr int kExactOverlapBodies = 7;   // bodies per block with kOverlap
+constexpr int kExactBodies = 32;         // without
+constexpr int kExactTerms = 2 * 4 * kExactOverlapBodies * 97;
+
+struct ExactSm {
+  double t[kExactTerms];  // [buffer][component][body][tile j, padded by one]
+  double x[6][kExactBodies];
+  unsigned long long q[kExactBodies];
+  int i[kExactBodies];
+};
+static_assert(4 * kExactBodies * 33 <= kExactTerms, "term buffer");
+
+struct F64J {
+  double x, y, z, u, v, w, m;
+};
+
+__device__ __forceinline__ F64J load_f64_j(const ForceArgs& A, int j) {
+  F64J J = {};
+  if (j < A.n)
+    J = F64J{A.x[0][j], A.x[1][j], A.x[2][j], A.w[0][j],
+             A.w[1][j], A.w[2][j], A.m[j]};
+  return J;
+}
+
+// the larger of q and x as bit patterns of doubles, where q >= 0; like
+// `if (x > q) q = x`, which a NaN or a negative x leaves alone (integer
+// operations: an FP64 comparison would take the FP64 pipe)
+__device__ __forceinline__ unsigned long long max_bits(unsigned long long q,
+                                                       double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return b <= 0x7ff0000000000000ULL && b > q ? b : q;
+}
+
+// active bodies k0 .. k0 + B - 1 of the list
+template <bool kOverlap>
+__device__ void f64_exact_group(const ForceArgs& A, int n_act, int k0, int B,
+                                ExactSm& sm) {
+  constexpr int TJ = kOverlap ? 96 : 32;           // j per tile
+  constexpr int TT = kOverlap ? 96 : kThreads;     // threads forming terms
+  constexpr int RB = TT / TJ;                      // bodies side by side
+  constexpr int NB = kOverlap ? kExactOverlapBodies : kExactBodies / RB;
+  constexpr int SB = TJ + 1;                       // stride of a body's terms
+  constexpr int SC = (kOverlap ? kExactOverlapBodies : kExactBodies) * SB;
+  const int t = threadIdx.x, lane = t & 31;
   const double eps2 = A.eps2;
-  F64Acc s = {0.0, 0.0, 0.0, 0.0, 0.0};
-  double ql = 0.0;
-  for (int jt = 0; jt < A.n; jt += kThreads) {
-    const int j = jt + t;
-    double tx = 0.0, ty = 0.0, tz = 0.0, tp = 0.0;
-    if (j < A.n && j != i) {
-      const double dx = __dsub_rn(A.x[0][j], xi);
-      const double dy = __dsub_rn(A.x[1][j], yi);
-      const double dz = __dsub_rn(A.x[2][j], zi);
-      const double s2 = __dadd_rn(
-          __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                    __dmul_rn(dz, dz)),
-          eps2);
-      const double sq = __dsqrt_rn(s2);
-      const double mj = A.m[j];
-      const double f = __ddiv_rn(mj, __dmul_rn(s2, sq));
-      tx = __dmul_rn(f, dx);
-      ty = __dmul_rn(f, dy);
-      tz = __dmul_rn(f, dz);
-      tp = __ddiv_rn(mj, sq);
-      const double wx = __dsub_rn(A.w[0][j], ui);
-      const double wy = __dsub_rn(A.w[1][j], vi);
-      const double wz = __dsub_rn(A.w[2][j], wi);
-      const double c = __ddiv_rn(
-          __dadd_rn(__dadd_rn(__dmul_rn(wx, wx), __dmul_rn(wy, wy)),
-                    __dmul_rn(wz, wz)),
-          s2);
-      if (c > ql) ql = c;
-      if (f > ql) ql = f;
+  __syncthreads();  // the previous group's use of sm is over
+  if (t < B) {
+    const int i = A.idx[k0 + t];
+    sm.i[t] = i;
+    for (int c = 0; c < 3; ++c) {
+      sm.x[c][t] = A.x[c][i];
+      sm.x[3 + c][t] = A.w[c][i];
     }
-    __syncthreads();  // the previous tile's terms have been added
-    red[0][t] = tx;
-    red[1][t] = ty;
-    red[2][t] = tz;
-    red[3][t] = tp;
-    __syncthreads();
-    if (t == 0) {
-      const int cnt = min(kThreads, A.n - jt);
-      for (int q = 0; q < cnt; ++q) {
-        s.ax = __dadd_rn(s.ax, red[0][q]);
-        s.ay = __dadd_rn(s.ay, red[1][q]);
-        s.az = __dadd_rn(s.az, red[2][q]);
-        s.ph = __dsub_rn(s.ph, red[3][q]);
+    sm.q[t] = 0;
+  }
+  __syncthreads();
+  const bool forms = !kOverlap || t >= 32;
+  const int tt = kOverlap ? t - 32 : t;
+  const int tj = tt % TJ, tb = tt / TJ;
+  // this lane's sum: body sb, component sc
+  const int sb = kOverlap ? lane >> 2 : lane;
+  const int sc = kOverlap ? lane & 3 : t >> 5;
+  const bool adds = (!kOverlap || t < 32) && sb < B;
+  double sum = 0.0;
+  unsigned long long q[NB];
+#pragma unroll
+  for (int e = 0; e < NB; ++e) q[e] = 0;
+
+  auto form = [&](int j, const F64J& J, double* T) {
+#pragma unroll
+    for (int e = 0; e < NB; ++e) {
+      const int b = tb + e * RB;
+      if (b >= B) break;
+      double tx = 0.0, ty = 0.0, tz = 0.0, tp = 0.0;
+      if (j < A.n && j != sm.i[b]) {
+        const double dx = __dsub_rn(J.x, sm.x[0][b]);
+        const double dy = __dsub_rn(J.y, sm.x[1][b]);
+        const double dz = __dsub_rn(J.z, sm.x[2][b]);
+        const double s2 = __dadd_rn(
+            __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
+                      __dmul_rn(dz, dz)),
+            eps2);
+        const double sq = __dsqrt_rn(s2);
+        const double f = __ddiv_rn(J.m, __dmul_rn(s2, sq));
+        tx = __dmul_rn(f, dx);
+        ty = __dmul_rn(f, dy);
+        tz = __dmul_rn(f, dz);
+        tp = __ddiv_rn(J.m, sq);
+        const double wx = __dsub_rn(J.u, sm.x[3][b]);
+        const double wy = __dsub_rn(J.v, sm.x[4][b]);
+        const double wz = __dsub_rn(J.w, sm.x[5][b]);
+        const double c = __ddiv_rn(
+            __dadd_rn(__dadd_rn(__dmul_rn(wx, wx), __dmul_rn(wy, wy)),
+                      __dmul_rn(wz, wz)),
+            s2);
+        q[e] = max_bits(max_bits(q[e], c), f);
       }
+      double* p = T + b * SB + tj;
+      p[0] = tx;
+      p[SC] = ty;
+      p[2 * SC] = tz;
+      p[3 * SC] = -tp;
+    }
+  };
+  auto add = [&](const double* T, int cnt) {
+    const double* p = T + sc * SC + sb * SB;
+    int e = 0;
+    for (; e + 8 <= cnt; e += 8) {
+      double y[8];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) y[w] = p[e + w];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) sum = __dadd_rn(sum, y[w]);
+    }
+    for (; e < cnt; ++e) sum = __dadd_rn(sum, p[e]);
+  };
+
+  const int tiles = (A.n + TJ - 1) / TJ;
+  F64J J = {};
+  if (forms) J = load_f64_j(A, tj);
+  for (int k = 0; k < tiles + (kOverlap ? 1 : 0); ++k) {
+    double* T = sm.t + (kOverlap ? (k & 1) * 4 * SC : 0);
+    if (forms && k < tiles) {
+      // the next tile's j are on their way while this tile's terms form
+      const F64J N = load_f64_j(A, (k + 1) * TJ + tj);
+      form(k * TJ + tj, J, T);
+      J = N;
+    }
+    if constexpr (kOverlap) {
+      if (adds && k > 0)
+        add(sm.t + ((k - 1) & 1) * 4 * SC, min(TJ, A.n - (k - 1) * TJ));
+      __syncthreads();
+    } else {
+      __syncthreads();
+      if (adds) add(T, min(TJ, A.n - k * TJ));
+      __syncthreads();
     }
   }
-  __syncthreads();
-  red[4][t] = ql;
-  __syncthreads();
-  for (int half = kThreads / 2; half >= 1; half >>= 1) {
-    if (t < half) red[4][t] = fmax(red[4][t], red[4][t + half]);
-    __syncthreads();
+  if (forms) {
+#pragma unroll
+    for (int e = 0; e < NB; ++e)
+      if (tb + e * RB < B && q[e]) atomicMax(&sm.q[tb + e * RB], q[e]);
   }
-  if (t == 0) write_partial(A, n_act, 0, k, s.ax, s.ay, s.az, s.ph, red[4][0]);
-  __syncthreads();  // red is reused by the block's next body
+  __syncthreads();
+  // (a buffer too small for the sums gets none, as in write_partial)
+  if (5LL * n_act > A.part_cap) return;
+  if (adds) A.part[(long long)sc * n_act + k0 + sb] = sum;
+  if (t < B)
+    A.part[4LL * n_act + k0 + t] = __longlong_as_double((long long)sm.q[t]);
+}
+
+// bodies per block for `bodies` active bodies on a device of `sms` SMs:
+// one block per SM while kOverlap can hold them (at 7 bodies per block the
+// two forms take as long), beyond that up to 32 in two blocks per SM
+__device__ __forceinline__ int exact_bodies(int bodies, int sms) {
+  const int b = (bodies + sms - 1) / sms;
+  if (b <= kExactOverlapBodies) return b < 1 ? 1 : b;
+  return min(kExactBodies, max(kExactOverlapBodies + 1,
+                               (bodies + 2 * sms - 1) / (2 * sms)));
 }
 
 template <int IG>

@@ -218,7 +218,7 @@ __device__ __forceinline__ Plan ens_plan_for(int n_act, int n, int exact,
   p.S = 1;
   p.chunk = (n + 1) & ~1;
   if (exact) {
-    p.ig = 128;
+    p.ig = exact;  // bodies per block (f64_exact_group)
     p.direct = 0;
   } else {
     int ig = 1;
@@ -265,7 +265,7 @@ __device__ __forceinline__ T block_scan(T x, T* wt) {
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
-    ens_plan_kernel(Ens E, Params P, int init) {
+    ens_plan_kernel(Ens E, Params P, int sms, int init) {
   Ctl* ctl = P.ctl;
   if (!init && ctl->done) return;
   __shared__ int wti[32];
@@ -273,8 +273,9 @@ __global__ void __launch_bounds__(kPlanThreads)
   __shared__ int c_items, c_nact;
   __shared__ long long c_part;
   __shared__ unsigned long long s_inter;
-  __shared__ int s_fallback;
+  __shared__ int s_fallback, s_active;
   if (threadIdx.x == 0) {
+    s_active = 0;
     c_items = 0;
     c_nact = 0;
     c_part = 0;
@@ -284,10 +285,14 @@ __global__ void __launch_bounds__(kPlanThreads)
   __syncthreads();
   // the step's total work sets the size of a work item
   for (int c = threadIdx.x; c < E.nc; c += blockDim.x)
-    if (E.tau_next[c] != LLONG_MAX && E.cnt[c] > 0)
+    if (E.tau_next[c] != LLONG_MAX && E.cnt[c] > 0) {
       atomicAdd(&s_inter, (unsigned long long)E.cnt[c] *
                               (unsigned long long)(E.off[c + 1] - E.off[c]));
+      if (P.exact) atomicAdd(&s_active, E.cnt[c]);
+    }
   __syncthreads();
+  // ascending-j sums: bodies per block for the active bodies of the step
+  const int exact = P.exact ? exact_bodies(s_active, sms) : 0;
   const unsigned long long total_w = s_inter;
   double per_item = (double)total_w / kEnsTargetItems;
   // the split partials of the step must fit the partial-sum buffer
@@ -299,7 +304,7 @@ __global__ void __launch_bounds__(kPlanThreads)
     for (int c = threadIdx.x; c < E.nc; c += blockDim.x) {
       if (E.tau_next[c] == LLONG_MAX) continue;
       const int na = E.cnt[c];
-      const Plan p = ens_plan_for(na, E.off[c + 1] - E.off[c], P.exact,
+      const Plan p = ens_plan_for(na, E.off[c + 1] - E.off[c], exact,
                                   per_item);
       atomicAdd(&s_parts, 5ULL * p.S * (unsigned long long)na);
     }
@@ -317,7 +322,7 @@ __global__ void __launch_bounds__(kPlanThreads)
     if (valid) {
       nb = E.off[c + 1] - E.off[c];
       if (E.tau_next[c] != LLONG_MAX) n_act = E.cnt[c];
-      const Plan p = ens_plan_for(n_act, nb, P.exact, per_item);
+      const Plan p = ens_plan_for(n_act, nb, exact, per_item);
       E.plan[c] = p;
       items = n_act ? p.n_g * p.S : 0;
       parts = n_act ? 5LL * p.S * n_act : 0;
@@ -445,15 +450,15 @@ __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
   }
 }
 
+// FP64 work items with sums in any order (kExact = false: f64_item) or in
+// ascending j (true: f64_exact_group, whose shared memory is dynamic)
+template <bool kExact>
 __global__ void __launch_bounds__(kThreads)
-    ens_force_fp64_kernel(Bodies B, Ens E, const Ctl* ctl, double* part,
-                          int exact) {
+    ens_force_fp64_kernel(Bodies B, Ens E, const Ctl* ctl, double* part) {
   if (ctl->done) return;
   const int total = E.totals[0];
   if (total <= 0) return;
   __shared__ int s_off[kEnsMaxClusters + 1];
-  __shared__ F64Tile T;
-  __shared__ double red[5][kThreads];
   for (int c = threadIdx.x; c <= E.nc; c += blockDim.x) s_off[c] = E.item_off[c];
   __syncthreads();
   __shared__ int s_next;
@@ -463,18 +468,30 @@ __global__ void __launch_bounds__(kThreads)
     const int c = find_cluster(s_off, E.nc, w);
     const Plan p = E.plan[c];
     const int local = w - s_off[c];
-    const int g = local / p.S, split = local - (local / p.S) * p.S;
     const int n_act = E.cnt[c];
-    const ForceArgs A = cluster_args(B, E, c, part, p, n_act, exact);
-    switch (p.ig) {
-      case 128: f64_item<128>(A, n_act, p, g, split, T, red); break;
-      case 64: f64_item<64>(A, n_act, p, g, split, T, red); break;
-      case 32: f64_item<32>(A, n_act, p, g, split, T, red); break;
-      case 16: f64_item<16>(A, n_act, p, g, split, T, red); break;
-      case 8: f64_item<8>(A, n_act, p, g, split, T, red); break;
-      case 4: f64_item<4>(A, n_act, p, g, split, T, red); break;
-      case 2: f64_item<2>(A, n_act, p, g, split, T, red); break;
-      default: f64_item<1>(A, n_act, p, g, split, T, red); break;
+    const ForceArgs A = cluster_args(B, E, c, part, p, n_act, kExact);
+    if constexpr (kExact) {
+      extern __shared__ __align__(16) unsigned char s_dyn[];
+      ExactSm& sm = *reinterpret_cast<ExactSm*>(s_dyn);
+      const int k0 = local * p.ig, nb = min(p.ig, n_act - k0);
+      if (p.ig <= kExactOverlapBodies)
+        f64_exact_group<true>(A, n_act, k0, nb, sm);
+      else
+        f64_exact_group<false>(A, n_act, k0, nb, sm);
+    } else {
+      __shared__ F64Tile T;
+      __shared__ double red[5][kThreads];
+      const int g = local / p.S, split = local - (local / p.S) * p.S;
+      switch (p.ig) {
+        case 128: f64_item<128>(A, n_act, p, g, split, T, red); break;
+        case 64: f64_item<64>(A, n_act, p, g, split, T, red); break;
+        case 32: f64_item<32>(A, n_act, p, g, split, T, red); break;
+        case 16: f64_item<16>(A, n_act, p, g, split, T, red); break;
+        case 8: f64_item<8>(A, n_act, p, g, split, T, red); break;
+        case 4: f64_item<4>(A, n_act, p, g, split, T, red); break;
+        case 2: f64_item<2>(A, n_act, p, g, split, T, red); break;
+        default: f64_item<1>(A, n_act, p, g, split, T, red); break;
+      }
     }
   }
 }
@@ -605,9 +622,14 @@ ForceLaunch ens_force_launch_shape(int precision, int device) {
         &per_sm, ens_force_mixed_kernel, kThreads, 0);
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, ens_force_fp64_kernel, kThreads, 0);
+        &per_sm, ens_force_fp64_kernel<false>, kThreads, 0);
+  if (sms < 1) sms = 1;
+  cudaFuncSetAttribute(ens_force_fp64_kernel<true>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)sizeof(ExactSm));
   ForceLaunch fl;
-  fl.grid = (sms < 1 ? 1 : sms) * (per_sm < 1 ? 1 : per_sm);
+  fl.grid = sms * (per_sm < 1 ? 1 : per_sm);
+  fl.exact_grid = 2 * sms;
   fl.threads = kThreads;
   fl.tile_i = kThreads;
   fl.part_cap = 0;
@@ -634,6 +656,19 @@ void launch_ens_pass_setup(const Bodies& B, const Params& P, const Ens& E,
                                                                   cur);
 }
 
+static void launch_ens_force(const Bodies& B, const Params& P, const Ens& E,
+                             const ForceLaunch& fl, int precision, int exact,
+                             cudaStream_t s) {
+  if (precision)
+    ens_force_mixed_kernel<<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl, B.part);
+  else if (exact)
+    ens_force_fp64_kernel<true><<<fl.exact_grid, kThreads, sizeof(ExactSm),
+                                  s>>>(B, E, P.ctl, B.part);
+  else
+    ens_force_fp64_kernel<false><<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl,
+                                                              B.part);
+}
+
 void launch_ens_step(const Bodies& B, const Params& P, const Ens& E,
                      const History& HA, const History& HB,
                      const ForceLaunch& fl, int precision, int exact,
@@ -642,13 +677,9 @@ void launch_ens_step(const Bodies& B, const Params& P, const Ens& E,
   ens_select_kernel<<<blocks_for(E.nc, 4, 1 << 20), 128, 0, s>>>(E, P);
   ens_predict_kernel<<<blocks_for(B.n, 64, 1 << 30), 64, 0, s>>>(B, P, E,
                                                                  HB);
-  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, 0);
+  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, fl.exact_grid / 2, 0);
   if (ev0) cudaEventRecordWithFlags(ev0, s, evflags);
-  if (precision)
-    ens_force_mixed_kernel<<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl, B.part);
-  else
-    ens_force_fp64_kernel<<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl, B.part,
-                                                       exact);
+  launch_ens_force(B, P, E, fl, precision, exact, s);
   if (ev1) cudaEventRecordWithFlags(ev1, s, evflags);
   ens_correct_kernel<<<blocks_for(B.n, 64, 1 << 20), 64, 0, s>>>(B, P, E, HA,
                                                                  HB, B.part);
@@ -658,12 +689,8 @@ void launch_ens_init(const Bodies& B, const Params& P, const Ens& E,
                      const ForceLaunch& fl, int precision, int exact,
                      cudaStream_t s) {
   ens_init_active_kernel<<<blocks_for(B.n, 256, 4096), 256, 0, s>>>(E, B.n);
-  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, 1);
-  if (precision)
-    ens_force_mixed_kernel<<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl, B.part);
-  else
-    ens_force_fp64_kernel<<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl, B.part,
-                                                       exact);
+  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, fl.exact_grid / 2, 1);
+  launch_ens_force(B, P, E, fl, precision, exact, s);
   ens_init_finalize_kernel<<<blocks_for(B.n, 256, 4096), 256, 0, s>>>(
       B, P, E, B.part);
 }

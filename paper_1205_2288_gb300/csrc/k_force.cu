@@ -40,10 +40,7 @@ namespace tsbts {
 Plan plan_force(int precision, int exact, int n_act, int n, int grid,
                 long long part_cap) {
   Plan best = {kThreads, (n_act + kThreads - 1) / kThreads, 1, n};
-  // ascending-j sums: one body per block while the bodies fit the grid
-  // (latency-bound: the block computes the terms, one thread adds them),
-  // one body per thread beyond that (throughput-bound)
-  if (exact && n_act > 0 && n_act <= grid) return Plan{1, n_act, 1, n, 0};
+  // ascending-j sums have one split and take no plan (force_exact_kernel)
   if (exact || n_act <= 0) return best;
   const int lane_min = precision ? kLaneMinMix : kLaneMinF64;
   double best_cost = 1e300;
@@ -73,17 +70,9 @@ Plan plan_force(int precision, int exact, int n_act, int n, int grid,
 }
 
 __device__ __forceinline__ Plan make_plan(int n_act, int n, int grid,
-                                          int exact, long long part_cap,
-                                          int lane_min, int tile) {
+                                          long long part_cap, int lane_min) {
   Plan p;
   p.direct = 0;
-  if (exact) {
-    p.ig = n_act <= grid ? 1 : kThreads;
-    p.n_g = (n_act + p.ig - 1) / p.ig;
-    p.S = 1;
-    p.chunk = n;
-    return p;
-  }
   // Narrow the i-groups until about kSplitCap splits fill the grid: j-lanes
   // inside a block are combined by a cheap shared-memory tree, whereas
   // every extra split adds a partial sum that the consumer must read.
@@ -105,7 +94,6 @@ __device__ __forceinline__ Plan make_plan(int n_act, int n, int grid,
   p.n_g = n_g;
   p.S = S;
   p.chunk = chunk;
-  (void)tile;
   return p;
 }
 
@@ -136,8 +124,7 @@ __device__ __forceinline__ Plan launch_plan(const ForceArgs& A,
     return p;
   }
   if (A.plans) return A.plans[n_act];
-  return make_plan(n_act, A.n, gridDim.x, precision ? 0 : A.exact,
-                   A.part_cap, lane_min, precision ? kTileMix : kTileF64);
+  return make_plan(n_act, A.n, gridDim.x, A.part_cap, lane_min);
 }
 
 // Launch prologue shared by both precisions: wait for the prediction
@@ -162,12 +149,6 @@ __global__ void __launch_bounds__(kThreads)
     *A.nsplit_out = P.S;
   __shared__ F64Tile T;
   __shared__ double red[5][kThreads];
-  if (A.exact && P.ig == 1) {
-    // few bodies, ascending-j sums: one body per block
-    for (int w = blockIdx.x; w < n_act; w += gridDim.x)
-      f64_item_exact1(A, n_act, w, red);
-    return;
-  }
   switch (P.ig) {
     case 128: f64_items<128>(A, n_act, P, T, red); break;
     case 64: f64_items<64>(A, n_act, P, T, red); break;
@@ -177,6 +158,23 @@ __global__ void __launch_bounds__(kThreads)
     case 4: f64_items<4>(A, n_act, P, T, red); break;
     case 2: f64_items<2>(A, n_act, P, T, red); break;
     default: f64_items<1>(A, n_act, P, T, red); break;
+  }
+}
+
+// FP64 with ascending-j sums (f64_exact_group), two blocks per SM
+__global__ void __launch_bounds__(kThreads)
+    force_exact_kernel(const __grid_constant__ ForceArgs A) {
+  int n_act = 0;
+  if (!force_prologue(A, n_act)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && A.nsplit_out) *A.nsplit_out = 1;
+  __shared__ ExactSm sm;
+  const int B = exact_bodies(n_act, gridDim.x / 2);
+  for (int k0 = blockIdx.x * B; k0 < n_act; k0 += gridDim.x * B) {
+    const int nb = min(B, n_act - k0);
+    if (B <= kExactOverlapBodies)
+      f64_exact_group<true>(A, n_act, k0, nb, sm);
+    else
+      f64_exact_group<false>(A, n_act, k0, nb, sm);
   }
 }
 
@@ -284,6 +282,7 @@ ForceLaunch force_launch_shape(int precision, int device) {
   if (per_sm < 1) per_sm = 1;
   ForceLaunch fl;
   fl.grid = sms * per_sm;
+  fl.exact_grid = 2 * sms;
   fl.threads = kThreads;
   fl.tile_i = kThreads;
   fl.part_cap = 5LL * fl.grid * kThreads;
@@ -313,6 +312,10 @@ cudaError_t launch_force(int precision, const ForceArgs& fa,
   cfg.numAttrs = pdl ? 1 : 0;
   if (precision)
     return cudaLaunchKernelEx(&cfg, force_mixed_kernel, fa, pt ? *pt : none);
+  if (fa.exact) {
+    cfg.gridDim = dim3(fl.exact_grid);
+    return cudaLaunchKernelEx(&cfg, force_exact_kernel, fa);
+  }
   return cudaLaunchKernelEx(&cfg, force_fp64_kernel, fa, pt ? *pt : none);
 }
 
