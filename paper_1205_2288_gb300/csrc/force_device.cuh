@@ -56,33 +56,59 @@ struct __align__(16) F64Tile {
 };
 
 struct F64Acc {
-  double ax, ay, az, ph, q;
+  double ax, ay, az, ph;
 };
 
-// 1/sqrt(s2) in FP64 for the j-split path: the FP32 reciprocal square root
-// refined by two Newton-Raphson steps for 1/sqrt (y <- y + y (1 - s2 y^2)/2,
-// each squaring the relative error: 2^-22 -> 2^-44 -> below FP64 rounding),
-// ten FP64 operations instead of a correctly rounded square root and
-// division (the FP64 pipe of this GPU is narrow). s2 outside 1e-36 .. 1e36
-// takes the correctly rounded form.
-__device__ __forceinline__ double rsqrt_f64(double s2) {
-  if (!(s2 > 1e-36 && s2 < 1e36)) return __ddiv_rn(1.0, __dsqrt_rn(s2));
-  double y = (double)rsqrtf((float)s2);
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double e = fma(-(s2 * y), y, 1.0);
-    y = fma(0.5 * y, e, y);
-  }
+// 1/sqrt(x) of a normal x (relative error about 2^-22; a subnormal x, which
+// no caller passes, would count as 0)
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
-// The same pair term with the reciprocal square root and fused
-// multiply-adds (j-split path: the sums are not in the oracle's order
-// anyway, and each term agrees with the rounded definition to ~1e-16).
+// 1/sqrt(s2) in FP64 for the j-split path: the FP32 reciprocal square root y
+// (2^-22 relative) and one third-order step for y^-2 = s2 (Householder):
+// with e = 1 - s2 y^2, y <- y + y e (1/2 + 3 e / 8), whose error is
+// 5 e^3 / 16 < 2^-62. The FP64 pipe of this GPU is narrow (a warp's FP64
+// instruction takes 64 cycles) and the integer pipe is idle, so the
+// conversions to and from FP32 and the range test are integer operations on
+// the exponent fields (the significand is cut, not rounded: another 2^-24 in
+// y), which leaves five FP64 operations. s2 outside 2^-119 .. 2^119 (and
+// NaN) takes the correctly rounded form.
+__device__ __forceinline__ double rsqrt_f64(double s2) {
+  const int hi = __double2hiint(s2), lo = __double2loint(s2);
+  if ((unsigned)hi - 0x38800000u >= 0x0ee00000u)
+    return __ddiv_rn(1.0, __dsqrt_rn(s2));
+  const float f = __uint_as_float(
+      __funnelshift_l((unsigned)lo, (unsigned)hi - 0x38000000u, 3));
+  const unsigned r = __float_as_uint(rsqrt_ftz(f));
+  const double y = __hiloint2double((int)((r >> 3) + 0x38000000u),
+                                    (int)(r << 29));
+  const double e = fma(-(s2 * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// the larger of q and x as bit patterns of doubles, where q >= 0; like
+// `if (x > q) q = x`, which a NaN or a negative x leaves alone (integer
+// operations: an FP64 comparison would take the FP64 pipe)
+__device__ __forceinline__ unsigned long long max_bits(unsigned long long q,
+                                                       double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return b <= 0x7ff0000000000000ULL && b > q ? b : q;
+}
+
+// One pair term with the reciprocal square root and fused multiply-adds
+// (the sums are not in the oracle's order anyway, and each term agrees with
+// the rounded definition to ~1e-16): 25 FP64 operations. The maximum of the
+// criterion is taken on the bit patterns (q). With the FP64 conversions,
+// range test and comparisons and two second-order steps it was 37; 5000 of
+// 20000 bodies went from 7.30 to 5.85 ms.
 __device__ __forceinline__ void pair_f64_fast(const F64Tile& T, int t,
                                               double xi, double yi, double zi,
                                               double ui, double vi, double wi,
-                                              double eps2, F64Acc& s) {
+                                              double eps2, F64Acc& s,
+                                              unsigned long long& q) {
   const double dx = T.x[t] - xi;
   const double dy = T.y[t] - yi;
   const double dz = T.z[t] - zi;
@@ -99,7 +125,7 @@ __device__ __forceinline__ void pair_f64_fast(const F64Tile& T, int t,
   const double wy = T.v[t] - vi;
   const double wz = T.w[t] - wi;
   const double c = fma(wx, wx, fma(wy, wy, wz * wz)) * rinv2;
-  s.q = fmax(s.q, fmax(c, f));
+  q = max_bits(max_bits(q, c), f);
 }
 
 template <int IG>
@@ -123,7 +149,8 @@ __device__ void f64_item(const ForceArgs& A, int n_act, const Plan& P,
       vi = A.w[1][i];
       wi = A.w[2][i];
     }
-    F64Acc s = {0.0, 0.0, 0.0, 0.0, 0.0};
+    F64Acc s = {0.0, 0.0, 0.0, 0.0};
+    unsigned long long qb = 0;
     const int j0 = split * P.chunk;
     const int j1 = min(A.n, j0 + P.chunk);
     for (int jt = j0; jt < j1; jt += TJ) {
@@ -142,15 +169,16 @@ __device__ void f64_item(const ForceArgs& A, int n_act, const Plan& P,
       __syncthreads();
       for (int q = jl; q < cnt; q += JG) {
         if (jt + q == i) continue;
-        pair_f64_fast(T, q, xi, yi, zi, ui, vi, wi, eps2, s);
+        pair_f64_fast(T, q, xi, yi, zi, ui, vi, wi, eps2, s, qb);
       }
     }
+    double qm = __longlong_as_double((long long)qb);
     if constexpr (JG > 1) {
       red[0][t] = s.ax;
       red[1][t] = s.ay;
       red[2][t] = s.az;
       red[3][t] = s.ph;
-      red[4][t] = s.q;
+      red[4][t] = qm;
       __syncthreads();
       for (int half = JG / 2; half >= 1; half >>= 1) {
         if (jl < half) {
@@ -165,11 +193,11 @@ __device__ void f64_item(const ForceArgs& A, int n_act, const Plan& P,
         s.ay = red[1][t];
         s.az = red[2][t];
         s.ph = red[3][t];
-        s.q = red[4][t];
+        qm = red[4][t];
       }
     }
     if (jl == 0 && valid)
-      write_partial(A, n_act, split, k, s.ax, s.ay, s.az, s.ph, s.q);
+      write_partial(A, n_act, split, k, s.ax, s.ay, s.az, s.ph, qm);
   }
 }
 
@@ -219,15 +247,6 @@ __device__ __forceinline__ F64J load_f64_j(const ForceArgs& A, int j) {
     J = F64J{A.x[0][j], A.x[1][j], A.x[2][j], A.w[0][j],
              A.w[1][j], A.w[2][j], A.m[j]};
   return J;
-}
-
-// the larger of q and x as bit patterns of doubles, where q >= 0; like
-// `if (x > q) q = x`, which a NaN or a negative x leaves alone (integer
-// operations: an FP64 comparison would take the FP64 pipe)
-__device__ __forceinline__ unsigned long long max_bits(unsigned long long q,
-                                                       double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  return b <= 0x7ff0000000000000ULL && b > q ? b : q;
 }
 
 // active bodies k0 .. k0 + B - 1 of the list
