@@ -217,10 +217,10 @@ double* const* fsum_of(AdjCtx& A) {
 // own kernel and the reverse sweep's work splits)
 void choose_plans(tsbts_ctx* c, AdjCtx& A) {
   (void)c;
-  A.plan_init = plan_force(A.mixed, A.exact, A.n, A.n, A.fl.grid, A.part_cap);
+  A.plan_init = plan_force(A.mixed, A.exact, A.n, A.n, A.fl, A.part_cap);
   for (long long s = 0; s < A.S; ++s)
     A.plans[s] = plan_force(A.mixed, A.exact, (int)(A.off[s + 1] - A.off[s]),
-                            A.n, A.fl.grid, A.part_cap);
+                            A.n, A.fl, A.part_cap);
 }
 
 // The pass p seen by the kernels, with record cursor `cur` (forward or

@@ -137,8 +137,8 @@ void build_plan_table(tsbts_ctx* c) {
   c->pt = PlanTable{};
   c->pt.nb = (int)b.size();
   for (size_t k = 0; k < b.size(); ++k)
-    c->pt.b[k] = plan_force(c->cfg.precision, c->exact, b[k], c->n,
-                            c->fl.grid, c->B.part_cap);
+    c->pt.b[k] = plan_force(c->cfg.precision, c->exact, b[k], c->n, c->fl,
+                            c->B.part_cap);
 }
 
 // one block step: A (select + predict), B (force), C (correct). Plain
@@ -665,8 +665,8 @@ int init_common(tsbts_ctx* c, int64_t n, const double* m, const double* r,
       fa.n_act_ptr = nullptr;
       fa.nsplit_out = c->d_nsplit;
       fa.done = nullptr;
-      fa.plan = plan_force(c->cfg.precision, c->exact, c->n, c->n,
-                           c->fl.grid, c->B.part_cap);
+      fa.plan = plan_force(c->cfg.precision, c->exact, c->n, c->n, c->fl,
+                           c->B.part_cap);
       fa.has_plan = 1;
       ck(launch_force(c->cfg.precision, fa, c->fl, c->s), "init force");
       launch_init_finalize(c->B, P, c->d_nsplit, c->s);
@@ -1226,7 +1226,7 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
     fa.eps2f = (float)(eps * eps);
     fa.exact = precision == TSBTS_FP64 &&
                (exact_order == 1 || (exact_order < 0 && n <= 8192));
-    fa.plan = plan_force(precision, fa.exact, (int)n_act, ni, fl.grid,
+    fa.plan = plan_force(precision, fa.exact, (int)n_act, ni, fl,
                          S.part_cap);
     if (precision == TSBTS_MIXED && ni <= (1 << 20)) {
       // measured plans: the first call for a new n tunes them on these j
@@ -1404,7 +1404,7 @@ extern "C" int tsbts_force_static(int precision, int exact_order, int64_t n,
   fa.eps2f = (float)(eps * eps);
   fa.exact = precision == TSBTS_FP64 &&
              (exact_order == 1 || (exact_order < 0 && n <= 8192));
-  fa.plan = plan_force(precision, fa.exact, (int)n_act, ni, fl.grid,
+  fa.plan = plan_force(precision, fa.exact, (int)n_act, ni, fl,
                        kStaticPartDoubles);
   fa.has_plan = 1;
   e = launch_force(precision, fa, fl, s);

@@ -32,17 +32,21 @@
 namespace tsbts {
 
 // Host choice of the work plan for n_act active bodies: over i-group widths
-// IG = 128 .. 1 and split counts S = 1 .. kSplitCap, minimise a cost model
-// of waves of the grid times the per-item time (j per thread plus a fixed
-// item overhead and the block's reduction tree) plus the consumer's cost of
-// reading S partial sums. Wave quantisation is what the search is for: 256
-// items on a 456-block grid leave 44% of the GPU idle.
-Plan plan_force(int precision, int exact, int n_act, int n, int grid,
-                long long part_cap) {
-  Plan best = {kThreads, (n_act + kThreads - 1) / kThreads, 1, n};
+// IG = 128 .. 1 and split counts S, minimise the time of the busiest block
+// (mixed) or SM (FP64) plus the consumer's cost of reading S partial sums.
+// Wave quantisation is what the search is for: 256 items on a 456-block grid
+// leave 44% of the GPU idle. The FP64 pipe is saturated by one block per SM,
+// so an SM's time is its number of items, whatever the number of resident
+// blocks: 640 items on 152 SMs cost five items' time, not 4.2 (5000 of 20000
+// bodies: 5.85 ms with S chosen for the waves of the resident grid, 4.93 ms
+// by items per SM).
+Plan plan_force(int precision, int exact, int n_act, int n,
+                const ForceLaunch& fl, long long part_cap) {
+  Plan best = {kThreads, (n_act + kThreads - 1) / kThreads, 1, n, 0};
   // ascending-j sums have one split and take no plan (force_exact_kernel)
   if (exact || n_act <= 0) return best;
   const int lane_min = precision ? kLaneMinMix : kLaneMinF64;
+  const int cap = precision ? kSplitCap : 2 * kSplitCap;
   double best_cost = 1e300;
   for (int ig = kThreads; ig >= 1; ig >>= 1) {
     if (ig > 2 * n_act && ig > 1) continue;
@@ -51,18 +55,25 @@ Plan plan_force(int precision, int exact, int n_act, int n, int grid,
     while ((1 << lg) < jg) ++lg;
     const long long n_g = (n_act + ig - 1) / ig;
     long long smax = n / ((long long)jg * lane_min);
-    smax = std::max<long long>(1, std::min<long long>(smax, kSplitCap));
+    smax = std::max<long long>(1, std::min<long long>(smax, cap));
     for (int S = 1; S <= smax; ++S) {
       if (S > 1 && (long long)S * 5 * n_act > part_cap) break;
       long long chunk = (n + S - 1) / S;
-      chunk = (chunk + 1) & ~1LL;
       const long long items = n_g * S;
-      const long long waves = (items + grid - 1) / grid;
-      const double per_item = (double)((chunk + jg - 1) / jg) + 96.0 + 8.0 * lg;
-      const double cost = waves * per_item + 16.0 * S * (1 + n_act / 4096);
+      double cost;
+      if (precision) {
+        chunk = (chunk + 1) & ~1LL;
+        const long long waves = (items + fl.grid - 1) / fl.grid;
+        const double per_item =
+            (double)((chunk + jg - 1) / jg) + 96.0 + 8.0 * lg;
+        cost = waves * per_item + 16.0 * S * (1 + n_act / 4096);
+      } else {
+        const long long per_sm = (items + fl.sms - 1) / fl.sms;
+        cost = per_sm * ((double)((chunk + jg - 1) / jg) + 2.0) + 0.3 * S;
+      }
       if (cost < best_cost) {
         best_cost = cost;
-        best = Plan{ig, (int)n_g, S, (int)chunk};
+        best = Plan{ig, (int)n_g, S, (int)chunk, 0};
       }
     }
   }
@@ -282,6 +293,7 @@ ForceLaunch force_launch_shape(int precision, int device) {
   if (per_sm < 1) per_sm = 1;
   ForceLaunch fl;
   fl.grid = sms * per_sm;
+  fl.sms = sms;
   fl.exact_grid = 2 * sms;
   fl.threads = kThreads;
   fl.tile_i = kThreads;

@@ -372,6 +372,7 @@ __device__ inline double history_dts_at(const History& H, int start, int end,
 // grid size and threads of the force kernels on the current device
 struct ForceLaunch {
   int grid;
+  int sms;
   int exact_grid;      // blocks of the FP64 kernel with ascending-j sums
   int threads;
   int tile_i;          // active bodies per work item
@@ -384,8 +385,8 @@ ForceLaunch force_launch_shape(int precision, int device);
 // at least the grid's own floor). Every caller of one body count uses the
 // same capacity, so plans tuned by one fit the buffers of another.
 long long force_partial_capacity(const ForceLaunch& fl, long long n);
-Plan plan_force(int precision, int exact, int n_act, int n, int grid,
-                long long part_cap);
+Plan plan_force(int precision, int exact, int n_act, int n,
+                const ForceLaunch& fl, long long part_cap);
 // measured plans of the mixed force kernel per active count 0..n (cached
 // per device, n and grid for the life of the process)
 const std::vector<Plan>* tuned_plans(int device, int n, int grid);
