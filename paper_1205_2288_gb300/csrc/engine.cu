@@ -117,7 +117,6 @@ ForceArgs force_args_engine(tsbts_ctx* c, int p) {
   fa.eps2 = c->eps * c->eps;
   fa.eps2f = (float)(c->eps * c->eps);
   fa.exact = c->exact;
-  fa.plans = nullptr;
   return fa;
 }
 

@@ -11,26 +11,81 @@ namespace tsbts {
 
 constexpr int kThreads = 128;   // threads per block
 constexpr int kTileF64 = 64;    // j per shared-memory tile, FP64
-constexpr int kTileMix = 256;   // j per shared-memory tile, mixed
+constexpr int kTileMix = 512;   // j per shared-memory tile, mixed
+constexpr int kStrip = 256;     // j per thread between two folds, mixed
 constexpr int kLaneMinMix = 16; // fewest j per thread in a split item
 constexpr int kLaneMinF64 = 8;
-constexpr int kSplitCap = 16;   // most j-splits of one active body
+constexpr int kSplitCap = 16;   // most j-splits of one of many active bodies
+constexpr int kSplitCapFew = 64;  // ... of one of at most kFewBodies
+constexpr int kFewBodies = 512;
 constexpr int kSplitCapDirect = 128;  // most j-splits of a direct-load plan
 constexpr int kDirectBatch = 4;  // j records per lane loaded in one batch
+constexpr int kMixMaxGroup = 2 * kThreads;  // bodies of a tiled mixed item
+constexpr int kMixMinBlocks = 3;  // register budget of the mixed kernels
 
-// tuning of the mixed pair loop (compile-time; defaults measured on GB300)
-#ifndef TSBTS_MIX_UNROLL
-#define TSBTS_MIX_UNROLL 4
-#endif
-#ifndef TSBTS_MIX_QUAD
-#define TSBTS_MIX_QUAD 1
-#endif
-#ifndef TSBTS_MIX_MINB
-#define TSBTS_MIX_MINB 3
-#endif
-constexpr int kMixUnroll = TSBTS_MIX_UNROLL;  // unroll of the j-pair loop
-constexpr bool kMixQuad = TSBTS_MIX_QUAD;     // 128-bit loads of four j
-constexpr int kMixMinBlocks = TSBTS_MIX_MINB; // register budget hint
+// Tiled plan for n_act active bodies: over the group widths 256 .. 8 and
+// over w = 1 .. 5 waves of the grid, take the largest split count S whose
+// items fit w waves, and rate it by the waves its items take times the time
+// of an item, in quads of j per lane. Sharing a tile among fewer bodies
+// makes a quad dearer (staging, distinct shared loads: measured at 131072 j
+// 1163, 1123, 1057 and 960 G interactions/s with 256, 128, 64 and 32 bodies
+// per item: + 1/40 per lane of a body); an item's own cost (loading its
+// bodies, combining and writing sums) counts as kItemQuads. On a grid of 456
+// blocks this fills more than 95% of the last wave for nearly every count;
+// one width and split count per power of two of n_act took 40 groups of 128
+// bodies (5000 of 20000) at 59%, 184 us per call instead of 122.
+constexpr int kItemQuads = 12;
+constexpr int kTiledTries = 6 * 5;  // widths x wave counts, at most 32
+
+__host__ __device__ inline Plan tiled_try(int k, int n_act, int n, int grid,
+                                          long long part_cap, float* cost) {
+  const int jg = 1 << (k % 6), w = k / 6 + 1;
+  const int ig = kMixMaxGroup / jg;
+  const unsigned n_g = (unsigned)(n_act + ig - 1) / ig;
+  const unsigned quads = (unsigned)(n + 3) / 4;
+  unsigned smax = quads / (jg * (kLaneMinMix / 4));
+  const unsigned cap = n_act <= kFewBodies ? kSplitCapFew : kSplitCap;
+  if (smax > cap) smax = cap;
+  if ((long long)smax * 5 * n_act > part_cap)
+    smax = (unsigned)(part_cap / (5LL * n_act));
+  unsigned S = (unsigned)(grid * w) / n_g;
+  if (S > smax) S = smax;
+  if (S < 1) S = 1;
+  const unsigned waves = (n_g * S + grid - 1) / grid;
+  const unsigned lane = (quads + S * jg - 1) / (S * jg);
+  *cost = (float)waves * ((float)lane * (1.f + 0.025f * jg) + kItemQuads);
+  return Plan{ig, (int)n_g, (int)S, (int)(4 * ((quads + S - 1) / S)), 0};
+}
+
+inline Plan tiled_plan(int n_act, int n, int grid, long long part_cap) {
+  Plan best{};
+  float best_cost = 3e38f;
+  for (int k = 0; k < kTiledTries; ++k) {
+    float c;
+    const Plan p = tiled_try(k, n_act, n, grid, part_cap, &c);
+    if (c < best_cost) {
+      best_cost = c;
+      best = p;
+    }
+  }
+  return best;
+}
+
+// the same on the device, lane k rating try k
+__device__ __forceinline__ Plan tiled_plan_warp(int n_act, int n, int grid,
+                                                long long part_cap) {
+  const int lane = threadIdx.x & 31;
+  float c;
+  Plan p = tiled_try(lane < kTiledTries ? lane : 0, n_act, n, grid, part_cap,
+                     &c);
+  const unsigned key = (__float_as_uint(c) & ~31u) | (unsigned)lane;
+  const int src = (int)(__reduce_min_sync(kFull, key) & 31u);
+  p.ig = __shfl_sync(kFull, p.ig, src);
+  p.n_g = __shfl_sync(kFull, p.n_g, src);
+  p.S = __shfl_sync(kFull, p.S, src);
+  p.chunk = __shfl_sync(kFull, p.chunk, src);
+  return p;
+}
 
 __device__ __forceinline__ void write_partial(const ForceArgs& A, int n_act,
                                               int split, int k, double ax,
@@ -386,16 +441,34 @@ __device__ void f64_items(const ForceArgs& A, int n_act, const Plan& P,
 
 // ---------------------------------------------------------------------
 // Mixed: FP32 pair terms on double-single relative coordinates
-// d = (x_hi,j - x_hi,i) + (x_lo,j - x_lo,i); FP32 sums per j tile folded
-// into hi/lo compensated accumulators; q is an exact FP32 max.
+// d = (x_hi,j - x_hi,i) + (x_lo,j - x_lo,i); FP32 sums over kStrip j per
+// thread folded into hi/lo compensated accumulators; q is an exact FP32 max.
+//
+// What bounds the pair loop: an interaction is 26 FMA-pipe operations, in
+// packed f32x2 instructions of two pipe cycles each, so 26 pipe cycles per
+// warp; and those instructions and the two maxima read about 57 registers
+// per interaction, of which a scheduler reads two per cycle (packed FMAs of
+// three distinct operands, or packed adds beside maxima, measure 2/3 of the
+// pipe's rate), so about 28 cycles are the floor of this form.
+//  - Each thread holds two bodies: a register that holds a component of j
+//    and a 128-bit shared load of four of them serve twice as many
+//    interactions.
+//  - The reciprocal square root is the form that flushes subnormals, three
+//    instructions fewer than rsqrtf: s^2 >= eps^2 is a normal float, and
+//    then both give the same bits (kSafe: rsqrtf).
+//  - With JG > 1, JG neighbouring lanes share two bodies and take the j
+//    quads in turn; their sums are combined by shuffles.
+// All 131072 bodies: 14.8 ms (1163 G interactions/s, 34 cycles each), 16.3
+// ms before; the same with one body per thread: 16.1 ms.
 // ---------------------------------------------------------------------
 // structure of arrays: consecutive j pair up for f32x2. The tile is read
-// with 8- and 16-byte shared loads, so it must start on a 16-byte boundary
+// with 16-byte shared loads, so it must start on a 16-byte boundary
 // wherever the kernel places it among its other shared variables.
+template <int TJ>
 struct __align__(16) MixTile {
-  float xh[kTileMix], yh[kTileMix], zh[kTileMix], m[kTileMix];
-  float xl[kTileMix], yl[kTileMix], zl[kTileMix];
-  float u[kTileMix], v[kTileMix], w[kTileMix];
+  float xh[TJ], yh[TJ], zh[TJ], m[TJ];
+  float xl[TJ], yl[TJ], zl[TJ];
+  float u[TJ], v[TJ], w[TJ];
 };
 
 struct MixI {
@@ -431,29 +504,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
-__device__ __forceinline__ void pair_mixed(const MixI& I, const MixTile& T,
-                                           int t, float eps2, float& ax,
-                                           float& ay, float& az, float& ph,
-                                           float& q) {
-  const float dx = __fsub_rn(T.xh[t], I.xh) + __fsub_rn(T.xl[t], I.xl);
-  const float dy = __fsub_rn(T.yh[t], I.yh) + __fsub_rn(T.yl[t], I.yl);
-  const float dz = __fsub_rn(T.zh[t], I.zh) + __fsub_rn(T.zl[t], I.zl);
-  const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-  const float rinv = rsqrtf(s2);
-  const float rinv2 = rinv * rinv;
-  const float mr = T.m[t] * rinv;
-  const float mr3 = mr * rinv2;
-  ax = fmaf(mr3, dx, ax);
-  ay = fmaf(mr3, dy, ay);
-  az = fmaf(mr3, dz, az);
-  ph += mr;
-  const float wx = T.u[t] - I.u;
-  const float wy = T.v[t] - I.v;
-  const float wz = T.w[t] - I.w;
-  const float w2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
-  q = max3(q, w2 * rinv2, mr3);
-}
-
 // packed pairs of floats (two j per instruction)
 typedef unsigned long long f2;
 
@@ -485,27 +535,15 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-__device__ __forceinline__ f2 ld2(const float* p) {
-  return *reinterpret_cast<const f2*>(p);
-}
-
 // the j operands of two interactions, one packed pair per component
 struct J2 {
   f2 xh, yh, zh, m, xl, yl, zl, u, v, w;
 };
 
-// j = t, t + 1 (t even): one 64-bit shared load per component
-__device__ __forceinline__ J2 load_j2(const MixTile& T, int t) {
-  J2 J;
-  J.xh = ld2(&T.xh[t]); J.yh = ld2(&T.yh[t]); J.zh = ld2(&T.zh[t]);
-  J.m = ld2(&T.m[t]);
-  J.xl = ld2(&T.xl[t]); J.yl = ld2(&T.yl[t]); J.zl = ld2(&T.zl[t]);
-  J.u = ld2(&T.u[t]); J.v = ld2(&T.v[t]); J.w = ld2(&T.w[t]);
-  return J;
-}
-
 // j = t .. t + 3 (t a multiple of 4): one 128-bit shared load per component
-__device__ __forceinline__ void load_j4(const MixTile& T, int t, J2& a, J2& b) {
+template <int TJ>
+__device__ __forceinline__ void load_j4(const MixTile<TJ>& T, int t, J2& a,
+                                        J2& b) {
   const ulonglong2 xh = *reinterpret_cast<const ulonglong2*>(&T.xh[t]);
   const ulonglong2 yh = *reinterpret_cast<const ulonglong2*>(&T.yh[t]);
   const ulonglong2 zh = *reinterpret_cast<const ulonglong2*>(&T.zh[t]);
@@ -520,23 +558,32 @@ __device__ __forceinline__ void load_j4(const MixTile& T, int t, J2& a, J2& b) {
   b = J2{xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, u.y, v.y, w.y};
 }
 
+template <bool kSafe>
+__device__ __forceinline__ float rsqrt_of(float x) {
+  return kSafe ? rsqrtf(x) : rsqrt_ftz(x);
+}
+
+// eps^2 for which every s^2 is a normal float
+__device__ __forceinline__ bool normal_eps2(float eps2) {
+  return eps2 >= 1.17549435e-38f;
+}
+
 // two interactions (j = t, t + 1) on one body, all FMA-pipe work packed.
-// MASK: the pair with tile index `self` is the body itself; its 1/s is set
-// to 0, so it adds exact zeros and the sums equal those of the unmasked
-// loop over the other j.
-template <bool MASK>
+// kSafe: any s^2 >= 0 (rsqrtf), and the pair with tile index `self` is the
+// body itself: its 1/s is set to 0, so it adds exact zeros and the sums
+// equal those of the loop over the other j.
+template <bool kSafe>
 __device__ __forceinline__ void pair_mixed2(const f2 (&ii)[9], const J2& J,
-                                            int t, f2 eps2, f2& ax, f2& ay,
-                                            f2& az, f2& ph, float& q,
-                                            int self = -1) {
+                                            int t, f2 eps2, f2 (&s)[4],
+                                            float& q, int self = -1) {
   const f2 dx = add2(sub2(J.xh, ii[0]), sub2(J.xl, ii[3]));
   const f2 dy = add2(sub2(J.yh, ii[1]), sub2(J.yl, ii[4]));
   const f2 dz = add2(sub2(J.zh, ii[2]), sub2(J.zl, ii[5]));
   const f2 s2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, eps2)));
   float s0, s1;
   upk(s2, s0, s1);
-  float r0 = rsqrtf(s0), r1 = rsqrtf(s1);
-  if (MASK) {
+  float r0 = rsqrt_of<kSafe>(s0), r1 = rsqrt_of<kSafe>(s1);
+  if (kSafe) {
     if (t == self) r0 = 0.f;
     if (t + 1 == self) r1 = 0.f;
   }
@@ -544,10 +591,10 @@ __device__ __forceinline__ void pair_mixed2(const f2 (&ii)[9], const J2& J,
   const f2 rinv2 = mul2(rinv, rinv);
   const f2 mr = mul2(J.m, rinv);
   const f2 mr3 = mul2(mr, rinv2);
-  ax = fma2(mr3, dx, ax);
-  ay = fma2(mr3, dy, ay);
-  az = fma2(mr3, dz, az);
-  ph = add2(ph, mr);
+  s[0] = fma2(mr3, dx, s[0]);
+  s[1] = fma2(mr3, dy, s[1]);
+  s[2] = fma2(mr3, dz, s[2]);
+  s[3] = add2(s[3], mr);
   const f2 wx = sub2(J.u, ii[6]);
   const f2 wy = sub2(J.v, ii[7]);
   const f2 wz = sub2(J.w, ii[8]);
@@ -559,128 +606,175 @@ __device__ __forceinline__ void pair_mixed2(const f2 (&ii)[9], const J2& J,
   q = max3(max3(q, c0, m0), c1, m1);
 }
 
-template <int IG>
-__device__ __forceinline__ void finish_mixed_item(const ForceArgs& A,
-                                                  int n_act, int split, int k,
-                                                  bool valid, DS sx, DS sy,
-                                                  DS sz, DS sp, float q,
-                                                  float (*red)[kThreads]);
+// x as a double, by moving its exponent and significand (the FP64 pipe,
+// which a conversion would take, is 64 times narrower than the integer one)
+__device__ __forceinline__ double to_double(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+  if (e - 1u >= 254u) return (double)x;  // zero, subnormal, inf, NaN
+  return __hiloint2double(
+      (int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+      (int)(u << 29));
+}
 
-template <int IG>
-__device__ void mixed_item(const ForceArgs& A, int n_act, const Plan& P,
-    int g, int split, MixTile& T, float (*red)[kThreads]) {
-  constexpr int JG = kThreads / IG;
-  constexpr int TJ = kTileMix;
+__device__ __forceinline__ double to_double(DS a) {
+  return to_double(a.hi) + to_double(a.lo);
+}
+
+// Work item of the tiled plans: ig = 256 / JG active bodies against one
+// j-chunk, JG neighbouring lanes per pair of bodies (bodies il and
+// il + ig / 2 of the group). Lane jl takes the quads of j jl, jl + JG, ...
+// of each tile; a tile is filled up to a whole number of quads per lane with
+// massless j at a distance whose square overflows, which add exact zeros.
+// A body's own j is masked: while a tile is staged the warp ORs, over its
+// bodies, the positions in the lanes' quad order that hold one of them, and
+// only those iterations (and all of them where eps^2 is no normal float)
+// run the masked form. Both forms round alike, so a body's sums do not
+// depend on its warp-mates.
+template <int JG>
+__device__ __forceinline__ void mixed_item(const ForceArgs& A, int n_act,
+                                           const Plan& P, int g, int split,
+                                           MixTile<kTileMix>& T) {
+  constexpr int IG = kMixMaxGroup / JG;
+  constexpr int U = 2;                  // quads per lane and loop iteration
+  constexpr int kRound = 4 * JG * U;    // j of one iteration of the warp
+  constexpr int kIter = kStrip / 4;     // quads per lane between two folds
   const int t = threadIdx.x;
-  const int il = t % IG, jl = t / IG;
-  const float eps2 = A.eps2f;
-  {
-    const int k = g * IG + il;
-    const bool valid = k < n_act;
-    const int i = valid ? A.idx[k] : -1;
-    MixI I = {};
-    if (valid) {
-      const float4 h = A.jhi[i], l = A.jlo[i], vv = A.jv[i];
-      I.xh = h.x; I.yh = h.y; I.zh = h.z;
-      I.xl = l.x; I.yl = l.y; I.zl = l.z;
-      I.u = vv.x; I.v = vv.y; I.w = vv.z;
+  const int il = t / JG, jl = t % JG;
+  const float far = 1e30f;
+  int own[2];
+  f2 ii[2][9];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int k = g * IG + r * (IG / 2) + il;
+    own[r] = k < n_act ? A.idx[k] : -1;
+    float4 h = {}, l = {}, v = {};
+    if (own[r] >= 0) {
+      h = A.jhi[own[r]];
+      l = A.jlo[own[r]];
+      v = A.jv[own[r]];
     }
-    DS sx = {0, 0}, sy = {0, 0}, sz = {0, 0}, sp = {0, 0};
-    float q = 0.f;
-    const int j0 = split * P.chunk;
-    const int j1 = min(A.n, j0 + P.chunk);
-    // FP32 running sums over about kTileMix j per thread, then folded
-    float ax = 0, ay = 0, az = 0, ph = 0;
-    int tiles = 0;
-    for (int jt = j0; jt < j1; jt += TJ) {
-      const int cnt = min(TJ, j1 - jt);
-      __syncthreads();
-      for (int c = t; c < cnt; c += kThreads) {
-        const float4 h = A.jhi[jt + c], l = A.jlo[jt + c], vv = A.jv[jt + c];
-        T.xh[c] = h.x; T.yh[c] = h.y; T.zh[c] = h.z; T.m[c] = h.w;
-        T.xl[c] = l.x; T.yl[c] = l.y; T.zl[c] = l.z;
-        T.u[c] = vv.x; T.v[c] = vv.y; T.w[c] = vv.z;
+    ii[r][0] = pk(h.x, h.x); ii[r][1] = pk(h.y, h.y); ii[r][2] = pk(h.z, h.z);
+    ii[r][3] = pk(l.x, l.x); ii[r][4] = pk(l.y, l.y); ii[r][5] = pk(l.z, l.z);
+    ii[r][6] = pk(v.x, v.x); ii[r][7] = pk(v.y, v.y); ii[r][8] = pk(v.z, v.z);
+  }
+  DS s[2][4] = {};
+  float q[2] = {0.f, 0.f};
+  const f2 e2 = pk(A.eps2f, A.eps2f);
+  const bool all_safe = !normal_eps2(A.eps2f);
+  const int j0 = split * P.chunk;
+  const int j1 = min(A.n, j0 + P.chunk);
+  for (int jt = j0; jt < j1; jt += kTileMix) {
+    const int cnt = min(kTileMix, j1 - jt);
+    const int cntp = (cnt + kRound - 1) / kRound * kRound;
+    __syncthreads();
+#pragma unroll 2
+    for (int c = t; c < cntp; c += kThreads) {
+      float4 h = make_float4(far, far, far, 0.f), l = {}, v = {};
+      if (c < cnt) {
+        h = A.jhi[jt + c];
+        l = A.jlo[jt + c];
+        v = A.jv[jt + c];
       }
-      __syncthreads();
-      const bool self_here = valid && i >= jt && i < jt + cnt;
-      if (cnt == TJ) {
-        // thread jl takes the j pairs (2 jl, 2 jl + 1) + 2 JG m; a warp with
-        // a body inside the tile runs the same arithmetic with that pair
-        // masked, so each body's sums do not depend on its warp-mates
-        const f2 ii[9] = {pk(I.xh, I.xh), pk(I.yh, I.yh), pk(I.zh, I.zh),
-                          pk(I.xl, I.xl), pk(I.yl, I.yl), pk(I.zl, I.zl),
-                          pk(I.u, I.u),   pk(I.v, I.v),   pk(I.w, I.w)};
-        const f2 e2 = pk(eps2, eps2);
-        f2 pax = pk(0.f, 0.f), pay = pax, paz = pax, pph = pax;
-        const bool any_self = __any_sync(kFull, self_here);
-        const int sc = self_here ? i - jt : -1;
-        if constexpr (kMixQuad && 4 * JG <= TJ) {
-          // thread jl takes the j quads 4 jl + 4 JG m (128-bit loads)
-          if (any_self) {
-            for (int c = 4 * jl; c < TJ; c += 4 * JG) {
-              J2 a, b;
-              load_j4(T, c, a, b);
-              pair_mixed2<true>(ii, a, c, e2, pax, pay, paz, pph, q, sc);
-              pair_mixed2<true>(ii, b, c + 2, e2, pax, pay, paz, pph, q, sc);
-            }
-          } else {
-#pragma unroll kMixUnroll
-            for (int c = 4 * jl; c < TJ; c += 4 * JG) {
-              J2 a, b;
-              load_j4(T, c, a, b);
-              pair_mixed2<false>(ii, a, c, e2, pax, pay, paz, pph, q);
-              pair_mixed2<false>(ii, b, c + 2, e2, pax, pay, paz, pph, q);
+      T.xh[c] = h.x; T.yh[c] = h.y; T.zh[c] = h.z; T.m[c] = h.w;
+      T.xl[c] = l.x; T.yl[c] = l.y; T.zl[c] = l.z;
+      T.u[c] = v.x; T.v[c] = v.y; T.w[c] = v.z;
+    }
+    __syncthreads();
+    // this tile's position of each body's own j, and its quad number
+    // among this lane's (own_m < 0: not in the tile or another lane's)
+    int self[2], own_m[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      self[r] = own[r] >= jt && own[r] < jt + cnt ? own[r] - jt : -1;
+      own_m[r] = self[r] < 0 ? -1 : self[r] / (4 * JG);
+    }
+    const int iters = cntp / (4 * JG);
+    for (int m0 = 0; m0 < iters; m0 += kIter) {
+      unsigned lo = 0, hi = 0;
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const unsigned m = (unsigned)(own_m[r] - m0);
+        if (own_m[r] >= 0 && m < 32u) lo |= 1u << m;
+        if (own_m[r] >= 0 && m - 32u < 32u) hi |= 1u << (m - 32u);
+      }
+      lo = __reduce_or_sync(kFull, lo);
+      if (kTileMix / (4 * JG) > 32) hi = __reduce_or_sync(kFull, hi);
+      unsigned long long mask = ((unsigned long long)hi << 32) | lo;
+      if (all_safe) mask = ~0ULL;
+      const f2 z = pk(0.f, 0.f);
+      f2 p[2][4] = {{z, z, z, z}, {z, z, z, z}};
+      const int m1 = min(iters - m0, kIter);
+      for (int m = 0; m < m1; m += U, mask >>= U) {
+        const int c0 = 4 * (jl + JG * (m0 + m));
+        if ((mask & ((1ULL << U) - 1)) == 0) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            J2 a, b;
+            load_j4(T, c0 + 4 * JG * u, a, b);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              pair_mixed2<false>(ii[r], a, 0, e2, p[r], q[r]);
+              pair_mixed2<false>(ii[r], b, 0, e2, p[r], q[r]);
             }
           }
         } else {
-          if (any_self) {
-            for (int c = 2 * jl; c < TJ; c += 2 * JG)
-              pair_mixed2<true>(ii, load_j2(T, c), c, e2, pax, pay, paz, pph,
-                                q, sc);
-          } else {
-#pragma unroll kMixUnroll
-            for (int c = 2 * jl; c < TJ; c += 2 * JG)
-              pair_mixed2<false>(ii, load_j2(T, c), c, e2, pax, pay, paz, pph,
-                                 q);
+#pragma unroll 1
+          for (int u = 0; u < U; ++u) {
+            const int c = c0 + 4 * JG * u;
+            J2 a, b;
+            load_j4(T, c, a, b);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              pair_mixed2<true>(ii[r], a, c, e2, p[r], q[r], self[r]);
+              pair_mixed2<true>(ii[r], b, c + 2, e2, p[r], q[r], self[r]);
+            }
           }
         }
-        float a0, a1;
-        upk(pax, a0, a1);
-        ax += a0 + a1;
-        upk(pay, a0, a1);
-        ay += a0 + a1;
-        upk(paz, a0, a1);
-        az += a0 + a1;
-        upk(pph, a0, a1);
-        ph += a0 + a1;
-      } else {
-        for (int c = jl; c < cnt; c += JG) {
-          if (jt + c == i) continue;
-          pair_mixed(I, T, c, eps2, ax, ay, az, ph, q);
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          float a0, a1;
+          upk(p[r][c], a0, a1);
+          ds_add(s[r][c], a0 + a1);
         }
-      }
-      if (++tiles == JG) {
-        tiles = 0;
-        ds_add(sx, ax);
-        ds_add(sy, ay);
-        ds_add(sz, az);
-        ds_add(sp, ph);
-        ax = ay = az = ph = 0.f;
-      }
     }
-    ds_add(sx, ax);
-    ds_add(sy, ay);
-    ds_add(sz, az);
-    ds_add(sp, ph);
-    finish_mixed_item<IG>(A, n_act, split, k, valid, sx, sy, sz, sp, q, red);
+  }
+  // the JG lanes of a body pair: a butterfly, so every lane holds the sums
+#pragma unroll
+  for (int o = JG / 2; o >= 1; o >>= 1) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        ds_add(s[r][c], DS{__shfl_xor_sync(kFull, s[r][c].hi, o),
+                           __shfl_xor_sync(kFull, s[r][c].lo, o)});
+      q[r] = fmaxf(q[r], __shfl_xor_sync(kFull, q[r], o));
+    }
+  }
+  // lane r of a pair writes body r (one lane writes both when JG = 1)
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const bool second = JG > 1 ? jl == 1 : r == 1;
+    if (JG > 1 && (r == 1 || jl > 1)) break;
+    if ((second ? own[1] : own[0]) < 0) continue;
+    DS x[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      x[c] = DS{second ? s[1][c].hi : s[0][c].hi,
+                second ? s[1][c].lo : s[0][c].lo};
+    write_partial(A, n_act, split, g * IG + (second ? IG / 2 : 0) + il,
+                  to_double(x[0]), to_double(x[1]), to_double(x[2]),
+                  -to_double(x[3]), to_double(second ? q[1] : q[0]));
   }
 }
 
-template <int IG>
+template <int JG>
 __device__ void mixed_items(const ForceArgs& A, int n_act, const Plan& P,
-                            MixTile& T, float (*red)[kThreads]) {
+                            MixTile<kTileMix>& T) {
   for (int w = blockIdx.x; w < P.n_g * P.S; w += gridDim.x)
-    mixed_item<IG>(A, n_act, P, w / P.S, w % P.S, T, red);
+    mixed_item<JG>(A, n_act, P, w / P.S, w % P.S, T);
 }
 
 // Reduce the JG j-lane partial sums of each body in a fixed-order tree in
@@ -724,14 +818,13 @@ __device__ __forceinline__ void finish_mixed_item(const ForceArgs& A,
       }
     }
     if (jl == 0 && valid)
-      write_partial(A, n_act, split, k, (double)sx.hi + (double)sx.lo,
-                    (double)sy.hi + (double)sy.lo,
-                    (double)sz.hi + (double)sz.lo,
-                    -((double)sp.hi + (double)sp.lo), (double)q);
+      write_partial(A, n_act, split, k, to_double(sx), to_double(sy),
+                    to_double(sz), -to_double(sp), to_double(q));
     __syncthreads();  // red is reused by the next item
   }
 }
 
+template <bool kSafe>
 __device__ __forceinline__ void pair_mixed_g(const MixI& I, const float4 h,
                                              const float4 l, const float4 vv,
                                              float eps2, float& ax, float& ay,
@@ -740,7 +833,7 @@ __device__ __forceinline__ void pair_mixed_g(const MixI& I, const float4 h,
   const float dy = __fsub_rn(h.y, I.yh) + __fsub_rn(l.y, I.yl);
   const float dz = __fsub_rn(h.z, I.zh) + __fsub_rn(l.z, I.zl);
   const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-  const float rinv = rsqrtf(s2);
+  const float rinv = rsqrt_of<kSafe>(s2);
   const float rinv2 = rinv * rinv;
   const float mr = h.w * rinv;
   const float mr3 = mr * rinv2;
@@ -755,52 +848,35 @@ __device__ __forceinline__ void pair_mixed_g(const MixI& I, const float4 h,
   q = max3(q, w2 * rinv2, mr3);
 }
 
-// Narrow groups without shared-memory staging: j-lane jl of a body reads
-// j = j0 + jl, j0 + jl + JG, ... straight from global memory (the j records
-// are L2-resident), so a small active set costs no block-wide tile loads.
-// BATCH j records per lane are loaded in one batch before any is used, so
-// a small item waits for a few round trips to L2, not one per j; BATCH = 1
-// keeps the register budget of kernels that hold more state (ensembles).
-template <int IG, int BATCH = kDirectBatch>
-__device__ void mixed_direct_item(const ForceArgs& A, int n_act, const Plan& P,
-    int g, int split, float (*red)[kThreads]) {
-  constexpr int JG = kThreads / IG;
-  const int t = threadIdx.x;
-  const int il = t % IG, jl = t / IG;
+// The j sweep of a direct-load item: j-lane jl of a body reads
+// j = j0 + jl, j0 + jl + JG, ... straight from global memory.
+template <int JG, int BATCH, bool kSafe>
+__device__ __forceinline__ void direct_sweep(const ForceArgs& A,
+                                             const MixI& I, int i, int j0,
+                                             int jl, int j1, DS (&s)[4],
+                                             float& q) {
   const float eps2 = A.eps2f;
-  {
-    const int k = g * IG + il;
-    const bool valid = k < n_act;
-    const int i = valid ? A.idx[k] : -1;
-    MixI I = {};
-    if (valid) {
-      const float4 h = A.jhi[i], l = A.jlo[i], vv = A.jv[i];
-      I.xh = h.x; I.yh = h.y; I.zh = h.z;
-      I.xl = l.x; I.yl = l.y; I.zl = l.z;
-      I.u = vv.x; I.v = vv.y; I.w = vv.z;
-    }
-    DS sx = {0, 0}, sy = {0, 0}, sz = {0, 0}, sp = {0, 0};
-    float q = 0.f;
-    float ax = 0, ay = 0, az = 0, ph = 0;
-    const int j0 = split * P.chunk;
-    const int j1 = min(A.n, j0 + P.chunk);
-    int cnt = 0;
-    if constexpr (BATCH == 1) {
+  float ax = 0, ay = 0, az = 0, ph = 0;
+  auto fold = [&]() {
+    ds_add(s[0], ax);
+    ds_add(s[1], ay);
+    ds_add(s[2], az);
+    ds_add(s[3], ph);
+    ax = ay = az = ph = 0.f;
+  };
+  int cnt = 0;
+  if constexpr (BATCH == 1) {
 #pragma unroll 4
-      for (int j = j0 + jl; j < j1; j += JG) {
-        const float4 h = A.jhi[j], l = A.jlo[j], vv = A.jv[j];
-        if (j != i) pair_mixed_g(I, h, l, vv, eps2, ax, ay, az, ph, q);
-        if (++cnt == kTileMix) {
-          cnt = 0;
-          ds_add(sx, ax);
-          ds_add(sy, ay);
-          ds_add(sz, az);
-          ds_add(sp, ph);
-          ax = ay = az = ph = 0.f;
-        }
+    for (int j = j0 + jl; j < j1; j += JG) {
+      const float4 h = A.jhi[j], l = A.jlo[j], vv = A.jv[j];
+      if (j != i) pair_mixed_g<kSafe>(I, h, l, vv, eps2, ax, ay, az, ph, q);
+      if (++cnt == kStrip) {
+        cnt = 0;
+        fold();
       }
     }
-    for (int jb = j0 + jl; BATCH > 1 && jb < j1; jb += JG * BATCH) {
+  } else {
+    for (int jb = j0 + jl; jb < j1; jb += JG * BATCH) {
       float4 h[BATCH], l[BATCH], vv[BATCH];
 #pragma unroll
       for (int u = 0; u < BATCH; ++u) {
@@ -815,24 +891,49 @@ __device__ void mixed_direct_item(const ForceArgs& A, int n_act, const Plan& P,
       for (int u = 0; u < BATCH; ++u) {
         const int j = jb + u * JG;
         if (j < j1 && j != i)
-          pair_mixed_g(I, h[u], l[u], vv[u], eps2, ax, ay, az, ph, q);
+          pair_mixed_g<kSafe>(I, h[u], l[u], vv[u], eps2, ax, ay, az, ph, q);
       }
       cnt += BATCH;
-      if (cnt >= kTileMix) {
+      if (cnt >= kStrip) {
         cnt = 0;
-        ds_add(sx, ax);
-        ds_add(sy, ay);
-        ds_add(sz, az);
-        ds_add(sp, ph);
-        ax = ay = az = ph = 0.f;
+        fold();
       }
     }
-    ds_add(sx, ax);
-    ds_add(sy, ay);
-    ds_add(sz, az);
-    ds_add(sp, ph);
-    finish_mixed_item<IG>(A, n_act, split, k, valid, sx, sy, sz, sp, q, red);
   }
+  fold();
+}
+
+// Narrow groups without shared-memory staging (the j records are
+// L2-resident), so a small active set costs no block-wide tile loads.
+// BATCH j records per lane are loaded in one batch before any is used, so
+// a small item waits for a few round trips to L2, not one per j; BATCH = 1
+// keeps the register budget of kernels that hold more state (ensembles).
+template <int IG, int BATCH = kDirectBatch>
+__device__ void mixed_direct_item(const ForceArgs& A, int n_act, const Plan& P,
+    int g, int split, float (*red)[kThreads]) {
+  constexpr int JG = kThreads / IG;
+  const int t = threadIdx.x;
+  const int il = t % IG, jl = t / IG;
+  const int k = g * IG + il;
+  const bool valid = k < n_act;
+  const int i = valid ? A.idx[k] : -1;
+  MixI I = {};
+  if (valid) {
+    const float4 h = A.jhi[i], l = A.jlo[i], vv = A.jv[i];
+    I.xh = h.x; I.yh = h.y; I.zh = h.z;
+    I.xl = l.x; I.yl = l.y; I.zl = l.z;
+    I.u = vv.x; I.v = vv.y; I.w = vv.z;
+  }
+  DS s[4] = {};
+  float q = 0.f;
+  const int j0 = split * P.chunk;
+  const int j1 = min(A.n, j0 + P.chunk);
+  if (normal_eps2(A.eps2f))
+    direct_sweep<JG, BATCH, false>(A, I, i, j0, jl, j1, s, q);
+  else
+    direct_sweep<JG, BATCH, true>(A, I, i, j0, jl, j1, s, q);
+  finish_mixed_item<IG>(A, n_act, split, k, valid, s[0], s[1], s[2], s[3], q,
+                        red);
 }
 
 template <int IG>

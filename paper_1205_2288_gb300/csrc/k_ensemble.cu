@@ -412,13 +412,167 @@ __device__ __forceinline__ ForceArgs cluster_args(const Bodies& B,
   return A;
 }
 
-__global__ void __launch_bounds__(kThreads, kMixMinBlocks)
+constexpr int kEnsTile = 256;  // j per shared-memory tile
+
+// one interaction (tile slot t)
+template <bool kSafe>
+__device__ __forceinline__ void pair_mixed(const MixI& I,
+                                           const MixTile<kEnsTile>& T, int t,
+                                           float eps2, float& ax, float& ay,
+                                           float& az, float& ph, float& q) {
+  const float dx = __fsub_rn(T.xh[t], I.xh) + __fsub_rn(T.xl[t], I.xl);
+  const float dy = __fsub_rn(T.yh[t], I.yh) + __fsub_rn(T.yl[t], I.yl);
+  const float dz = __fsub_rn(T.zh[t], I.zh) + __fsub_rn(T.zl[t], I.zl);
+  const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
+  const float rinv = rsqrt_of<kSafe>(s2);
+  const float rinv2 = rinv * rinv;
+  const float mr = T.m[t] * rinv;
+  const float mr3 = mr * rinv2;
+  ax = fmaf(mr3, dx, ax);
+  ay = fmaf(mr3, dy, ay);
+  az = fmaf(mr3, dz, az);
+  ph += mr;
+  const float wx = T.u[t] - I.u;
+  const float wy = T.v[t] - I.v;
+  const float wz = T.w[t] - I.w;
+  const float w2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
+  q = max3(q, w2 * rinv2, mr3);
+}
+
+// Tiled work item of a cluster: IG active bodies, one per thread, JG = 128 /
+// IG threads sharing a body. The items are short (about 12000 interactions),
+// so what the single-system item gains with two bodies per thread it would
+// lose to its longer prologue. In a full tile thread jl takes the j quads
+// 4 jl + 4 JG m. A body's own j is masked: the warp ORs the loop iterations
+// that hold one of its bodies, and only those (and all of them where eps^2
+// is no normal float) run the masked form, which rounds like the other one,
+// so a body's sums do not depend on its warp-mates. (With the whole tile
+// masked whenever one of 32 bodies lay in it, most tiles of a partial
+// active set ran masked.)
+template <int IG>
+__device__ void ens_tiled_item(const ForceArgs& A, int n_act, const Plan& P,
+                               int g, int split, MixTile<kEnsTile>& T,
+                               float (*red)[kThreads]) {
+  constexpr int JG = kThreads / IG;
+  constexpr int TJ = kEnsTile;
+  constexpr int kIter = TJ / (4 * JG);  // quads per thread and tile
+  constexpr int U = 4 < kIter ? 4 : kIter;
+  static_assert(kIter <= 64 && kIter % U == 0, "iteration mask");
+  const int t = threadIdx.x;
+  const int il = t % IG, jl = t / IG;
+  const float eps2 = A.eps2f;
+  const bool normal = normal_eps2(eps2);
+  const int k = g * IG + il;
+  const bool valid = k < n_act;
+  const int i = valid ? A.idx[k] : -1;
+  MixI I = {};
+  if (valid) {
+    const float4 h = A.jhi[i], l = A.jlo[i], vv = A.jv[i];
+    I.xh = h.x; I.yh = h.y; I.zh = h.z;
+    I.xl = l.x; I.yl = l.y; I.zl = l.z;
+    I.u = vv.x; I.v = vv.y; I.w = vv.z;
+  }
+  DS sx = {0, 0}, sy = {0, 0}, sz = {0, 0}, sp = {0, 0};
+  float q = 0.f;
+  const int j0 = split * P.chunk;
+  const int j1 = min(A.n, j0 + P.chunk);
+  // FP32 running sums over about kEnsTile j per thread, then folded
+  float ax = 0, ay = 0, az = 0, ph = 0;
+  int tiles = 0;
+  for (int jt = j0; jt < j1; jt += TJ) {
+    const int cnt = min(TJ, j1 - jt);
+    __syncthreads();
+    for (int c = t; c < cnt; c += kThreads) {
+      const float4 h = A.jhi[jt + c], l = A.jlo[jt + c], vv = A.jv[jt + c];
+      T.xh[c] = h.x; T.yh[c] = h.y; T.zh[c] = h.z; T.m[c] = h.w;
+      T.xl[c] = l.x; T.yl[c] = l.y; T.zl[c] = l.z;
+      T.u[c] = vv.x; T.v[c] = vv.y; T.w[c] = vv.z;
+    }
+    __syncthreads();
+    if (cnt == TJ) {
+      const f2 ii[9] = {pk(I.xh, I.xh), pk(I.yh, I.yh), pk(I.zh, I.zh),
+                        pk(I.xl, I.xl), pk(I.yl, I.yl), pk(I.zl, I.zl),
+                        pk(I.u, I.u),   pk(I.v, I.v),   pk(I.w, I.w)};
+      const f2 e2 = pk(eps2, eps2);
+      const f2 z = pk(0.f, 0.f);
+      f2 p[4] = {z, z, z, z};
+      const int self = valid && i >= jt && i < jt + cnt ? i - jt : -1;
+      const int own = self < 0 ? -1 : self / (4 * JG);  // its iteration
+      unsigned long long mask = ~0ULL;
+      if (normal) {
+        const unsigned lo = __reduce_or_sync(
+            kFull, own >= 0 && own < 32 ? 1u << own : 0u);
+        unsigned hi = 0;
+        if (kIter > 32)
+          hi = __reduce_or_sync(kFull, own >= 32 ? 1u << (own - 32) : 0u);
+        mask = ((unsigned long long)hi << 32) | lo;
+      }
+      for (int m = 0; m < kIter; m += U, mask >>= U) {
+        const int c0 = 4 * (jl + JG * m);
+        if ((mask & ((1ULL << U) - 1)) == 0) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            J2 a, b;
+            load_j4(T, c0 + 4 * JG * u, a, b);
+            pair_mixed2<false>(ii, a, 0, e2, p, q);
+            pair_mixed2<false>(ii, b, 0, e2, p, q);
+          }
+        } else {
+#pragma unroll 1
+          for (int u = 0; u < U; ++u) {
+            const int c = c0 + 4 * JG * u;
+            J2 a, b;
+            load_j4(T, c, a, b);
+            pair_mixed2<true>(ii, a, c, e2, p, q, self);
+            pair_mixed2<true>(ii, b, c + 2, e2, p, q, self);
+          }
+        }
+      }
+      float a0, a1;
+      upk(p[0], a0, a1);
+      ax += a0 + a1;
+      upk(p[1], a0, a1);
+      ay += a0 + a1;
+      upk(p[2], a0, a1);
+      az += a0 + a1;
+      upk(p[3], a0, a1);
+      ph += a0 + a1;
+    } else if (normal) {
+      for (int c = jl; c < cnt; c += JG) {
+        if (jt + c == i) continue;
+        pair_mixed<false>(I, T, c, eps2, ax, ay, az, ph, q);
+      }
+    } else {
+      for (int c = jl; c < cnt; c += JG) {
+        if (jt + c == i) continue;
+        pair_mixed<true>(I, T, c, eps2, ax, ay, az, ph, q);
+      }
+    }
+    if (++tiles == JG) {
+      tiles = 0;
+      ds_add(sx, ax);
+      ds_add(sy, ay);
+      ds_add(sz, az);
+      ds_add(sp, ph);
+      ax = ay = az = ph = 0.f;
+    }
+  }
+  ds_add(sx, ax);
+  ds_add(sy, ay);
+  ds_add(sz, az);
+  ds_add(sp, ph);
+  finish_mixed_item<IG>(A, n_act, split, k, valid, sx, sy, sz, sp, q, red);
+}
+
+constexpr int kEnsMinBlocks = 4;  // register budget: 128 without spills
+
+__global__ void __launch_bounds__(kThreads, kEnsMinBlocks)
     ens_force_mixed_kernel(Bodies B, Ens E, const Ctl* ctl, double* part) {
   if (ctl->done) return;
   const int total = E.totals[0];
   if (total <= 0) return;
   __shared__ int s_off[kEnsMaxClusters + 1];
-  __shared__ MixTile T;
+  __shared__ MixTile<kEnsTile> T;
   __shared__ float red[9][kThreads];
   for (int c = threadIdx.x; c <= E.nc; c += blockDim.x) s_off[c] = E.item_off[c];
   __syncthreads();
@@ -442,9 +596,9 @@ __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
       }
     } else {
       switch (p.ig) {
-        case 128: mixed_item<128>(A, n_act, p, g, split, T, red); break;
-        case 64: mixed_item<64>(A, n_act, p, g, split, T, red); break;
-        default: mixed_item<32>(A, n_act, p, g, split, T, red); break;
+        case 128: ens_tiled_item<128>(A, n_act, p, g, split, T, red); break;
+        case 64: ens_tiled_item<64>(A, n_act, p, g, split, T, red); break;
+        default: ens_tiled_item<32>(A, n_act, p, g, split, T, red); break;
       }
     }
   }

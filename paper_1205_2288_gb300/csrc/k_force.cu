@@ -5,19 +5,20 @@
 //
 // Work decomposition (the GB300 analogue of the paper's Alg. 4 data/work
 // partition). A persistent grid walks work items (i-group, j-chunk). The
-// launch reads the active count from device memory and picks, on the
-// device, the i-group width IG (bodies per 128-thread block):
-//  - IG = 128: one body per thread, every thread sweeps the j-chunk (data
-//    partition); the mixed path runs two j per packed f32x2 instruction.
-//  - IG < 128 (fewer than 128 active bodies): 128 / IG threads share each
-//    body's j-chunk and their partial sums are combined by a fixed-order
-//    tree in shared memory (work partition inside a block).
+// launch reads the active count from device memory and takes, on the
+// device, the group width and the number of j-chunks:
+//  - wide groups: the lanes sweep the j-chunk for their own bodies (data
+//    partition); the mixed path holds two bodies per thread and runs two j
+//    per packed f32x2 instruction;
+//  - narrow groups (fewer active bodies): several lanes share each body's
+//    j-chunk and their partial sums are combined in a fixed order inside the
+//    block (work partition inside a block).
 // The j range is further split across blocks so that the grid stays full;
 // split partial sums go to a scratch buffer and are added in split order by
 // the consumer. Every order is fixed, so results are deterministic.
 //
-// j records are staged tile by tile in shared memory with coalesced loads
-// and read back as broadcasts; the pair loop is FMA-pipe bound.
+// j records are staged tile by tile in shared memory with coalesced loads;
+// the pair loop is FMA-pipe bound.
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -31,46 +32,33 @@
 
 namespace tsbts {
 
-// Host choice of the work plan for n_act active bodies: over i-group widths
-// IG = 128 .. 1 and split counts S, minimise the time of the busiest block
-// (mixed) or SM (FP64) plus the consumer's cost of reading S partial sums.
-// Wave quantisation is what the search is for: 256 items on a 456-block grid
-// leave 44% of the GPU idle. The FP64 pipe is saturated by one block per SM,
-// so an SM's time is its number of items, whatever the number of resident
-// blocks: 640 items on 152 SMs cost five items' time, not 4.2 (5000 of 20000
-// bodies: 5.85 ms with S chosen for the waves of the resident grid, 4.93 ms
-// by items per SM).
+// Host choice of the work plan for n_act active bodies: tiled_plan in the
+// mixed path; in FP64, over i-group widths 128 .. 1 and split counts,
+// minimise the time of the busiest SM plus the consumer's cost of reading S
+// partial sums. The FP64 pipe is saturated by one block per SM, so an SM's
+// time is its number of items, whatever the number of resident blocks: 640
+// items on 152 SMs cost five items' time, not 4.2 (5000 of 20000 bodies: 5.85
+// ms with S chosen for the waves of the resident grid, 4.93 ms by items per
+// SM).
 Plan plan_force(int precision, int exact, int n_act, int n,
                 const ForceLaunch& fl, long long part_cap) {
   Plan best = {kThreads, (n_act + kThreads - 1) / kThreads, 1, n, 0};
   // ascending-j sums have one split and take no plan (force_exact_kernel)
   if (exact || n_act <= 0) return best;
-  const int lane_min = precision ? kLaneMinMix : kLaneMinF64;
-  const int cap = precision ? kSplitCap : 2 * kSplitCap;
+  if (precision) return tiled_plan(n_act, n, fl.grid, part_cap);
   double best_cost = 1e300;
   for (int ig = kThreads; ig >= 1; ig >>= 1) {
     if (ig > 2 * n_act && ig > 1) continue;
     const int jg = kThreads / ig;
-    int lg = 0;
-    while ((1 << lg) < jg) ++lg;
     const long long n_g = (n_act + ig - 1) / ig;
-    long long smax = n / ((long long)jg * lane_min);
-    smax = std::max<long long>(1, std::min<long long>(smax, cap));
+    long long smax = n / ((long long)jg * kLaneMinF64);
+    smax = std::max<long long>(1, std::min<long long>(smax, 2 * kSplitCap));
     for (int S = 1; S <= smax; ++S) {
       if (S > 1 && (long long)S * 5 * n_act > part_cap) break;
-      long long chunk = (n + S - 1) / S;
-      const long long items = n_g * S;
-      double cost;
-      if (precision) {
-        chunk = (chunk + 1) & ~1LL;
-        const long long waves = (items + fl.grid - 1) / fl.grid;
-        const double per_item =
-            (double)((chunk + jg - 1) / jg) + 96.0 + 8.0 * lg;
-        cost = waves * per_item + 16.0 * S * (1 + n_act / 4096);
-      } else {
-        const long long per_sm = (items + fl.sms - 1) / fl.sms;
-        cost = per_sm * ((double)((chunk + jg - 1) / jg) + 2.0) + 0.3 * S;
-      }
+      const long long chunk = (n + S - 1) / S;
+      const long long per_sm = (n_g * S + fl.sms - 1) / fl.sms;
+      const double per_item = (double)((chunk + jg - 1) / jg) + 2.0;
+      const double cost = per_sm * per_item + 0.3 * S;
       if (cost < best_cost) {
         best_cost = cost;
         best = Plan{ig, (int)n_g, S, (int)chunk, 0};
@@ -80,62 +68,29 @@ Plan plan_force(int precision, int exact, int n_act, int n,
   return best;
 }
 
-__device__ __forceinline__ Plan make_plan(int n_act, int n, int grid,
-                                          long long part_cap, int lane_min) {
-  Plan p;
-  p.direct = 0;
-  // Narrow the i-groups until about kSplitCap splits fill the grid: j-lanes
-  // inside a block are combined by a cheap shared-memory tree, whereas
-  // every extra split adds a partial sum that the consumer must read.
-  long long want = (long long)kSplitCap * n_act / grid;
-  int ig = 1;
-  while (ig < kThreads && 2LL * ig <= want) ig <<= 1;
-  const int jg = kThreads / ig;
-  const int n_g = (n_act + ig - 1) / ig;
-  int S = grid / n_g;
-  int smax = n / (jg * lane_min);
-  if (smax > kSplitCap) smax = kSplitCap;
-  if (smax < 1) smax = 1;
-  if (S > smax) S = smax;
-  if (S < 1) S = 1;
-  while (S > 1 && (long long)S * 5 * n_act > part_cap) --S;
-  int chunk = (n + S - 1) / S;
-  chunk = (chunk + 1) & ~1;  // packed loops take j in pairs
-  p.ig = ig;
-  p.n_g = n_g;
-  p.S = S;
-  p.chunk = chunk;
-  return p;
-}
-
-// The plan of a launch: fixed by the caller, from the bucket table, from a
-// per-count table, or chosen on the device.
+// The plan of a launch: fixed by the caller or from the bucket table. A
+// bucket's plan was made for the bucket's largest count; a smaller count has
+// fewer groups, so its split count is chosen again (tiled: tiled_plan;
+// direct and FP64: as many as keep the grid full).
 __device__ __forceinline__ Plan launch_plan(const ForceArgs& A,
                                             const PlanTable& PT, int n_act,
-                                            int lane_min, int precision) {
+                                            int precision) {
   if (A.has_plan) return A.plan;
-  if (PT.nb > 0) {
-    Plan p = PT.b[plan_bucket(n_act, PT.nb)];
-    p.n_g = (n_act + p.ig - 1) / p.ig;
-    if (precision) {
-      // a bucket's plan was measured at the bucket's largest count; a
-      // smaller count has fewer i-groups, so more j-splits keep the grid
-      // full (within the per-lane work floor and the partial buffer)
-      const int jg = kThreads / p.ig;
-      const int cap = p.direct ? kSplitCapDirect : 2 * kSplitCap;
-      const int lane_min = p.direct ? 2 : kLaneMinMix;
-      int S = min((int)gridDim.x / p.n_g, cap);
-      S = min(S, max(1, A.n / (jg * lane_min)));
-      while (S > p.S && (long long)S * 5 * n_act > A.part_cap) --S;
-      if (S > p.S) {
-        p.S = S;
-        p.chunk = (((A.n + S - 1) / S) + 1) & ~1;
-      }
+  Plan p = PT.b[plan_bucket(n_act, PT.nb)];
+  if (precision && !p.direct)
+    return tiled_plan_warp(n_act, A.n, gridDim.x, A.part_cap);
+  p.n_g = (n_act + p.ig - 1) / p.ig;
+  if (precision) {
+    const int jg = kThreads / p.ig;
+    int S = min((int)gridDim.x / p.n_g, kSplitCapDirect);
+    S = min(S, max(1, A.n / (jg * 2)));
+    while (S > p.S && (long long)S * 5 * n_act > A.part_cap) --S;
+    if (S > p.S) {
+      p.S = S;
+      p.chunk = (((A.n + S - 1) / S) + 1) & ~1;
     }
-    return p;
   }
-  if (A.plans) return A.plans[n_act];
-  return make_plan(n_act, A.n, gridDim.x, A.part_cap, lane_min);
+  return p;
 }
 
 // Launch prologue shared by both precisions: wait for the prediction
@@ -155,7 +110,7 @@ __global__ void __launch_bounds__(kThreads)
                       const __grid_constant__ PlanTable PT) {
   int n_act = 0;
   if (!force_prologue(A, n_act)) return;
-  const Plan P = launch_plan(A, PT, n_act, kLaneMinF64, 0);
+  const Plan P = launch_plan(A, PT, n_act, 0);
   if (blockIdx.x == 0 && threadIdx.x == 0 && A.nsplit_out)
     *A.nsplit_out = P.S;
   __shared__ F64Tile T;
@@ -194,10 +149,10 @@ __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
                        const __grid_constant__ PlanTable PT) {
   int n_act = 0;
   if (!force_prologue(A, n_act)) return;
-  const Plan P = launch_plan(A, PT, n_act, kLaneMinMix, 1);
+  const Plan P = launch_plan(A, PT, n_act, 1);
   if (blockIdx.x == 0 && threadIdx.x == 0 && A.nsplit_out)
     *A.nsplit_out = P.S;
-  __shared__ MixTile T;
+  __shared__ MixTile<kTileMix> T;
   __shared__ float red[9][kThreads];
   if (P.direct && P.ig <= 32) {
     // direct loads serve the narrow groups
@@ -212,14 +167,12 @@ __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
     return;
   }
   switch (P.ig) {
-    case 128: mixed_items<128>(A, n_act, P, T, red); break;
-    case 64: mixed_items<64>(A, n_act, P, T, red); break;
-    case 32: mixed_items<32>(A, n_act, P, T, red); break;
-    case 16: mixed_items<16>(A, n_act, P, T, red); break;
-    case 8: mixed_items<8>(A, n_act, P, T, red); break;
-    case 4: mixed_items<4>(A, n_act, P, T, red); break;
-    case 2: mixed_items<2>(A, n_act, P, T, red); break;
-    default: mixed_items<1>(A, n_act, P, T, red); break;
+    case 256: mixed_items<1>(A, n_act, P, T); break;
+    case 128: mixed_items<2>(A, n_act, P, T); break;
+    case 64: mixed_items<4>(A, n_act, P, T); break;
+    case 32: mixed_items<8>(A, n_act, P, T); break;
+    case 16: mixed_items<16>(A, n_act, P, T); break;
+    default: mixed_items<32>(A, n_act, P, T); break;
   }
 }
 
@@ -348,51 +301,44 @@ struct TuneKey {
 std::mutex g_tune_mu;
 std::map<TuneKey, std::vector<Plan>> g_tuned;
 
-// candidate plans for b active bodies: every i-group width, staged tiles for
-// the wider groups and direct loads for the narrower ones, split counts
-// {1, 2, 3, 4, 6, 8, 12, 16} within the per-thread work floor and the
-// partial-sum buffer, plus for each width the split count with the best
-// wave fill of the grid. Direct-load plans also try up to kSplitCapDirect
-// splits of a few j per lane: a small active set then spreads over the
+// candidate plans for b active bodies: the tiled one (tiled_plan; its width
+// and split count are chosen again for each count), and direct-load ones of
+// the narrower
+// groups with split counts {1, 2, 3, 4, 6, 8, ...} up to kSplitCapDirect and
+// the one that fills the waves of the grid best, within the per-thread work
+// floor and the partial-sum buffer: a small active set spreads over the
 // whole grid and each lane waits for one batch of loads.
 std::vector<Plan> candidates(int b, int n, int grid, long long part_cap) {
-  static const int kS[] = {1, 2, 3, 4, 6, 8, 12, 16};
-  static const int kSDirect[] = {24, 32, 48, 64, 96, 128};
+  static const int kS[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128};
   std::vector<Plan> out;
-  for (int ig = kThreads; ig >= 1; ig >>= 1) {
+  out.push_back(tiled_plan(b, n, grid, part_cap));
+  for (int ig = 32; ig >= 1; ig >>= 1) {
     if (ig > 2 * b && ig > 1) continue;
     const int jg = kThreads / ig;
     const int n_g = (b + ig - 1) / ig;
-    for (int direct = 0; direct <= 1; ++direct) {
-      if (direct && ig > 32) continue;
-      if (!direct && ig < 8) continue;
-      const int lane_min = direct ? 2 : kLaneMinMix;
-      const int cap = direct ? kSplitCapDirect : kSplitCap;
-      long long smax = n / ((long long)jg * lane_min);
-      smax = std::max<long long>(1, std::min<long long>(smax, cap));
-      std::vector<int> ss(std::begin(kS), std::end(kS));
-      if (direct) ss.insert(ss.end(), std::begin(kSDirect), std::end(kSDirect));
-      int best_s = 1;
-      double best_fill = 0;
-      for (int S = 1; S <= smax; ++S) {
-        const long long items = (long long)n_g * S;
-        const double fill =
-            (double)items / (double)(((items + grid - 1) / grid) * grid);
-        if (fill > best_fill + 1e-9) {
-          best_fill = fill;
-          best_s = S;
-        }
+    long long smax = n / ((long long)jg * 2);
+    smax = std::max<long long>(1, std::min<long long>(smax, kSplitCapDirect));
+    std::vector<int> ss(std::begin(kS), std::end(kS));
+    int best_s = 1;
+    double best_fill = 0;
+    for (int S = 1; S <= smax; ++S) {
+      const long long items = (long long)n_g * S;
+      const double fill =
+          (double)items / (double)(((items + grid - 1) / grid) * grid);
+      if (fill > best_fill + 1e-9) {
+        best_fill = fill;
+        best_s = S;
       }
-      ss.push_back(best_s);
-      std::sort(ss.begin(), ss.end());
-      ss.erase(std::unique(ss.begin(), ss.end()), ss.end());
-      for (int S : ss) {
-        if (S > smax) continue;
-        if ((long long)S * 5 * b > part_cap) continue;
-        long long chunk = (n + S - 1) / S;
-        chunk = (chunk + 1) & ~1LL;
-        out.push_back(Plan{ig, n_g, S, (int)chunk, direct});
-      }
+    }
+    ss.push_back(best_s);
+    std::sort(ss.begin(), ss.end());
+    ss.erase(std::unique(ss.begin(), ss.end()), ss.end());
+    for (int S : ss) {
+      if (S > smax) continue;
+      if ((long long)S * 5 * b > part_cap) continue;
+      long long chunk = (n + S - 1) / S;
+      chunk = (chunk + 1) & ~1LL;
+      out.push_back(Plan{ig, n_g, S, (int)chunk, 1});
     }
   }
   return out;
@@ -445,7 +391,6 @@ cudaError_t autotune_mixed_plans(int device, const ForceArgs& base,
       fa.n_act_ptr = nullptr;
       fa.nsplit_out = d_nsplit;
       fa.done = nullptr;
-      fa.plans = nullptr;
       fa.plan = p;
       fa.has_plan = 1;
       // the warm-up launch, timed, sets the batch: launches of more than
@@ -487,11 +432,15 @@ cudaError_t autotune_mixed_plans(int device, const ForceArgs& base,
                    n, buckets[bi], best[bi].ig, best[bi].S, best[bi].chunk,
                    best[bi].direct ? "direct" : "tiled", 1e3 * best_t[bi]);
   }
-  table->assign(n + 1, Plan{kThreads, 0, 1, n, 0});
+  table->assign(n + 1, Plan{kMixMaxGroup, 0, 1, n, 0});
   size_t bi = 0;
   for (int k = 1; k <= n; ++k) {
     while (buckets[bi] < k) ++bi;
     Plan p = best[bi];
+    if (!p.direct) {
+      (*table)[k] = tiled_plan(k, n, fl.grid, base.part_cap);
+      continue;
+    }
     p.n_g = (k + p.ig - 1) / p.ig;
     if ((long long)p.S * 5 * k > base.part_cap) {
       p.S = 1;

@@ -161,11 +161,12 @@ struct Ens {
   int* undone;
 };
 
-// Work plan of one force launch: IG active bodies per work item (128 / IG
-// threads per body), n_g i-groups, S j-splits of `chunk` j each; direct = 1
-// reads j records straight from global memory instead of staging tiles in
-// shared memory (for narrow groups, where a tile would be reused by few
-// bodies).
+// Work plan of one force launch: ig active bodies per work item (128 / ig
+// threads per body; tiled mixed items hold two bodies per thread, 256 / ig
+// threads per pair of bodies), n_g i-groups, S j-splits of `chunk` j each;
+// direct = 1 reads j records straight from global memory instead of staging
+// tiles in shared memory (for narrow groups, where a tile would be reused by
+// few bodies).
 struct Plan {
   int ig;
   int n_g;
@@ -177,7 +178,6 @@ struct Plan {
 // Arguments of the force kernels (shared by the integrator and the
 // stand-alone force entry point).
 struct ForceArgs {
-  const Plan* plans;   // plan per active count 0..n (nullable)
   Plan plan;           // used when has_plan
   int has_plan;
   int n;
