@@ -1251,7 +1251,8 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
                    fa.plan.n_g, fa.plan.S, fa.plan.chunk,
                    fa.plan.direct ? "direct" : "tiled");
     ck(launch_force(precision, fa, fl, s), "force");
-    ck(launch_force_finalize(S.part, S.nsplit, (int)n_act, a, phi, q, s),
+    ck(launch_force_finalize(S.part, fa.exact ? 1 : fa.plan.S, (int)n_act, a,
+                             phi, q, s),
        "force finalize");
     return TSBTS_OK;
   } catch (const CudaFail& f) {
@@ -1408,7 +1409,8 @@ extern "C" int tsbts_force_static(int precision, int exact_order, int64_t n,
   fa.has_plan = 1;
   e = launch_force(precision, fa, fl, s);
   if (e != cudaSuccess) return failed("force", e);
-  e = launch_force_finalize(part, nsplit, (int)n_act, a, phi, q, s);
+  e = launch_force_finalize(part, fa.exact ? 1 : fa.plan.S, (int)n_act, a,
+                            phi, q, s);
   if (e != cudaSuccess) return failed("force finalize", e);
   return TSBTS_OK;
 }

@@ -398,10 +398,10 @@ cudaError_t autotune_mixed_plans(int device, const ForceArgs& base,
 cudaError_t launch_force(int precision, const ForceArgs& fa,
                          const ForceLaunch& fl, cudaStream_t s,
                          const PlanTable* pt = nullptr, bool pdl = false);
-// sum nsplit partials per active body into AoS a, phi, q
-cudaError_t launch_force_finalize(const double* part, const int* nsplit,
-                                  int n_act, double* a, double* phi,
-                                  double* q, cudaStream_t s);
+// sum S split partials per active body into AoS a, phi, q
+cudaError_t launch_force_finalize(const double* part, int S, int n_act,
+                                  double* a, double* phi, double* q,
+                                  cudaStream_t s);
 // AoS (n, 3) -> packed j records for either precision
 cudaError_t launch_pack_aos(int precision, int n, const double* m,
                             const double* r, const double* v, double* sx,
