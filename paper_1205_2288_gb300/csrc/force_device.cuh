@@ -274,9 +274,8 @@ __device__ void f64_item(const ForceArgs& A, int n_act, const Plan& P,
 //    one body the block runs at the latency of the chain of n additions;
 //  - otherwise every warp forms terms, then warp c adds component c with
 //    one lane per body, so that up to 32 bodies share each addition.
-// Measured, 129 of 4099 bodies: 248 us; one thread adding all four sums of
-// one body (four instructions per j, on one pipe) took 698 us. The era of
-// Plummer 256 went from 184 to 92 ms. Without kOverlap the alternative is a
+// Measured, 129 of 4099 bodies: 159 us; one thread adding all four sums of
+// one body (four instructions per j, on one pipe) took 698 us. Without kOverlap the alternative is a
 // thread per body that forms and adds its terms, which does no more pairs
 // per FP64 instruction and leaves most of the chip idle at these counts.
 // ---------------------------------------------------------------------
@@ -375,17 +374,24 @@ __device__ void f64_exact_group(const ForceArgs& A, int n_act, int k0, int B,
       p[3 * SC] = -tp;
     }
   };
+  // the sums of a tile: 32 terms are fetched at once (waiting for eight at a
+  // time cost 16 cycles an addition), and as many eights added as hold
+  // terms; those past the end are zeros
   auto add = [&](const double* T, int cnt) {
     const double* p = T + sc * SC + sb * SB;
-    int e = 0;
-    for (; e + 8 <= cnt; e += 8) {
-      double y[8];
+#pragma unroll 1
+    for (int e = 0; e < cnt; e += 32) {
+      double y[32];
 #pragma unroll
-      for (int w = 0; w < 8; ++w) y[w] = p[e + w];
+      for (int w = 0; w < 32; ++w) y[w] = p[e + w];
 #pragma unroll
-      for (int w = 0; w < 8; ++w) sum = __dadd_rn(sum, y[w]);
+      for (int o = 0; o < 32; o += 8) {
+        if (e + o < cnt) {
+#pragma unroll
+          for (int w = 0; w < 8; ++w) sum = __dadd_rn(sum, y[o + w]);
+        }
+      }
     }
-    for (; e < cnt; ++e) sum = __dadd_rn(sum, p[e]);
   };
 
   const int tiles = (A.n + TJ - 1) / TJ;
@@ -422,14 +428,11 @@ __device__ void f64_exact_group(const ForceArgs& A, int n_act, int k0, int B,
     A.part[4LL * n_act + k0 + t] = __longlong_as_double((long long)sm.q[t]);
 }
 
-// bodies per block for `bodies` active bodies on a device of `sms` SMs:
-// one block per SM while kOverlap can hold them (at 7 bodies per block the
-// two forms take as long), beyond that up to 32 in two blocks per SM
+// bodies per block for `bodies` active bodies on a device of `sms` SMs, one
+// block per SM (two chains of additions on one SM share a scheduler's FP64
+// pipe: 129 blocks of a grid of two per SM took 246 us, of one per SM 170)
 __device__ __forceinline__ int exact_bodies(int bodies, int sms) {
-  const int b = (bodies + sms - 1) / sms;
-  if (b <= kExactOverlapBodies) return b < 1 ? 1 : b;
-  return min(kExactBodies, max(kExactOverlapBodies + 1,
-                               (bodies + 2 * sms - 1) / (2 * sms)));
+  return max(1, min(kExactBodies, (bodies + sms - 1) / sms));
 }
 
 template <int IG>

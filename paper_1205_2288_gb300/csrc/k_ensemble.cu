@@ -783,7 +783,7 @@ ForceLaunch ens_force_launch_shape(int precision, int device) {
                        (int)sizeof(ExactSm));
   ForceLaunch fl;
   fl.grid = sms * (per_sm < 1 ? 1 : per_sm);
-  fl.exact_grid = 2 * sms;
+  fl.sms = sms;
   fl.threads = kThreads;
   fl.tile_i = kThreads;
   fl.part_cap = 0;
@@ -816,8 +816,7 @@ static void launch_ens_force(const Bodies& B, const Params& P, const Ens& E,
   if (precision)
     ens_force_mixed_kernel<<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl, B.part);
   else if (exact)
-    ens_force_fp64_kernel<true><<<fl.exact_grid, kThreads, sizeof(ExactSm),
-                                  s>>>(B, E, P.ctl, B.part);
+    ens_force_fp64_kernel<true><<<fl.sms, kThreads, sizeof(ExactSm), s>>>(B, E, P.ctl, B.part);
   else
     ens_force_fp64_kernel<false><<<fl.grid, kThreads, 0, s>>>(B, E, P.ctl,
                                                               B.part);
@@ -831,7 +830,7 @@ void launch_ens_step(const Bodies& B, const Params& P, const Ens& E,
   ens_select_kernel<<<blocks_for(E.nc, 4, 1 << 20), 128, 0, s>>>(E, P);
   ens_predict_kernel<<<blocks_for(B.n, 64, 1 << 30), 64, 0, s>>>(B, P, E,
                                                                  HB);
-  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, fl.exact_grid / 2, 0);
+  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, fl.sms, 0);
   if (ev0) cudaEventRecordWithFlags(ev0, s, evflags);
   launch_ens_force(B, P, E, fl, precision, exact, s);
   if (ev1) cudaEventRecordWithFlags(ev1, s, evflags);
@@ -843,7 +842,7 @@ void launch_ens_init(const Bodies& B, const Params& P, const Ens& E,
                      const ForceLaunch& fl, int precision, int exact,
                      cudaStream_t s) {
   ens_init_active_kernel<<<blocks_for(B.n, 256, 4096), 256, 0, s>>>(E, B.n);
-  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, fl.exact_grid / 2, 1);
+  ens_plan_kernel<<<1, kPlanThreads, 0, s>>>(E, P, fl.sms, 1);
   launch_ens_force(B, P, E, fl, precision, exact, s);
   ens_init_finalize_kernel<<<blocks_for(B.n, 256, 4096), 256, 0, s>>>(
       B, P, E, B.part);

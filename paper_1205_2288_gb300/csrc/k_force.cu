@@ -127,14 +127,14 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// FP64 with ascending-j sums (f64_exact_group), two blocks per SM
+// FP64 with ascending-j sums (f64_exact_group), one block per SM
 __global__ void __launch_bounds__(kThreads)
     force_exact_kernel(const __grid_constant__ ForceArgs A) {
   int n_act = 0;
   if (!force_prologue(A, n_act)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0 && A.nsplit_out) *A.nsplit_out = 1;
   __shared__ ExactSm sm;
-  const int B = exact_bodies(n_act, gridDim.x / 2);
+  const int B = exact_bodies(n_act, gridDim.x);
   for (int k0 = blockIdx.x * B; k0 < n_act; k0 += gridDim.x * B) {
     const int nb = min(B, n_act - k0);
     if (B <= kExactOverlapBodies)
@@ -281,7 +281,7 @@ ForceLaunch force_launch_shape(int precision, int device) {
   ForceLaunch fl;
   fl.grid = sms * per_sm;
   fl.sms = sms;
-  fl.exact_grid = 2 * sms;
+
   fl.threads = kThreads;
   fl.tile_i = kThreads;
   fl.part_cap = 5LL * fl.grid * kThreads;
@@ -312,7 +312,7 @@ cudaError_t launch_force(int precision, const ForceArgs& fa,
   if (precision)
     return cudaLaunchKernelEx(&cfg, force_mixed_kernel, fa, pt ? *pt : none);
   if (fa.exact) {
-    cfg.gridDim = dim3(fl.exact_grid);
+    cfg.gridDim = dim3(fl.sms);
     return cudaLaunchKernelEx(&cfg, force_exact_kernel, fa);
   }
   return cudaLaunchKernelEx(&cfg, force_fp64_kernel, fa, pt ? *pt : none);

@@ -373,7 +373,6 @@ __device__ inline double history_dts_at(const History& H, int start, int end,
 struct ForceLaunch {
   int grid;
   int sms;
-  int exact_grid;      // blocks of the FP64 kernel with ascending-j sums
   int threads;
   int tile_i;          // active bodies per work item
   long long part_cap;  // doubles of partials the grid can produce
