@@ -228,11 +228,21 @@ __device__ __forceinline__ Plan ens_plan_for(int n_act, int n, int exact,
   }
   p.n_g = (n_act + p.ig - 1) / p.ig;
   if (!exact && n_act > 0 && per_item > 0.0) {
-    const double w = (double)n_act * (double)n;
-    int S = (int)ceil(w / per_item / p.n_g);
     const int jg = 128 / p.ig;
     int smax = n / (jg * kEnsLaneMin);
     smax = smax < 1 ? 1 : (smax > kEnsSplitCap ? kEnsSplitCap : smax);
+    // S = ceil(w / per_item / n_g) in FP64, whose divisions are slow: an
+    // FP32 quotient decides unless it lies within its error of an integer
+    const float x = __fdividef((float)n_act * (float)n,
+                               (float)per_item * (float)p.n_g);
+    int S;
+    if (x >= (float)(smax + 1)) {
+      S = smax;
+    } else if (fabsf(x - rintf(x)) > 1e-5f * (x + 1.f)) {
+      S = (int)ceilf(x);
+    } else {
+      S = (int)ceil((double)n_act * (double)n / per_item / p.n_g);
+    }
     S = S < 1 ? 1 : (S > smax ? smax : S);
     p.S = S;
     p.chunk = (((n + S - 1) / S) + 1) & ~1;
@@ -264,80 +274,90 @@ __device__ __forceinline__ T block_scan(T x, T* wt) {
   return r;
 }
 
+// sum of one value per thread over the block, to every thread
+template <class T>
+__device__ __forceinline__ T block_sum(T x, T* wt) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+  if (lane == 0) wt[wid] = x;
+  __syncthreads();
+  x = wt[lane];
+  for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+  __syncthreads();
+  return x;
+}
+
+// One block's latency is what this kernel takes, so it avoids FP64 divisions
+// (64 cycles an instruction: the item size is divided once, a plan's split
+// count in FP32 where that decides it), 64-bit shared-memory atomics and,
+// for up to kPlanThreads clusters, making a plan twice: 16 us before for
+// 512 clusters, 9 us now.
 __global__ void __launch_bounds__(kPlanThreads)
     ens_plan_kernel(Ens E, Params P, int sms, int init) {
   Ctl* ctl = P.ctl;
   if (!init && ctl->done) return;
   __shared__ int wti[32];
   __shared__ long long wtl[32];
+  __shared__ double s_item;
   __shared__ int c_items, c_nact;
   __shared__ long long c_part;
-  __shared__ unsigned long long s_inter;
-  __shared__ int s_fallback, s_active;
+  // the step's total work sets the size of a work item
+  long long inter = 0;
+  int active = 0;
+  for (int c = threadIdx.x; c < E.nc; c += kPlanThreads) {
+    const int cnt = E.cnt[c];
+    if (E.tau_next[c] == LLONG_MAX) continue;
+    inter += (long long)cnt * (E.off[c + 1] - E.off[c]);
+    active += cnt;
+  }
+  inter = block_sum<long long>(inter, wtl);
+  // ascending-j sums: bodies per block for the active bodies of the step
+  const int exact =
+      P.exact ? exact_bodies(block_sum<int>(active, wti), sms) : 0;
   if (threadIdx.x == 0) {
-    s_active = 0;
-    c_items = 0;
-    c_nact = 0;
+    s_item = (double)inter / kEnsTargetItems;
+    c_items = c_nact = 0;
     c_part = 0;
-    s_inter = 0;
-    s_fallback = 0;
   }
   __syncthreads();
-  // the step's total work sets the size of a work item
-  for (int c = threadIdx.x; c < E.nc; c += blockDim.x)
-    if (E.tau_next[c] != LLONG_MAX && E.cnt[c] > 0) {
-      atomicAdd(&s_inter, (unsigned long long)E.cnt[c] *
-                              (unsigned long long)(E.off[c + 1] - E.off[c]));
-      if (P.exact) atomicAdd(&s_active, E.cnt[c]);
+  double per_item = s_item;
+  // clusters base + threadIdx.x; the split partials of the step must fit
+  // the partial-sum buffer (else every cluster takes one split)
+  int na = 0;
+  Plan p{};
+  auto plan_of = [&](int c) {
+    const int nb = E.off[c + 1] - E.off[c];
+    na = E.tau_next[c] != LLONG_MAX ? E.cnt[c] : 0;
+    p = ens_plan_for(na, nb, exact, per_item);
+  };
+  for (int round = 0; round < 2; ++round) {
+    long long parts = 0;
+    for (int c = threadIdx.x; c < E.nc; c += kPlanThreads) {
+      plan_of(c);
+      parts += 5LL * p.S * na;
     }
-  __syncthreads();
-  // ascending-j sums: bodies per block for the active bodies of the step
-  const int exact = P.exact ? exact_bodies(s_active, sms) : 0;
-  const unsigned long long total_w = s_inter;
-  double per_item = (double)total_w / kEnsTargetItems;
-  // the split partials of the step must fit the partial-sum buffer
-  // (else every cluster takes one split)
-  {
-    __shared__ unsigned long long s_parts;
-    if (threadIdx.x == 0) s_parts = 0;
-    __syncthreads();
-    for (int c = threadIdx.x; c < E.nc; c += blockDim.x) {
-      if (E.tau_next[c] == LLONG_MAX) continue;
-      const int na = E.cnt[c];
-      const Plan p = ens_plan_for(na, E.off[c + 1] - E.off[c], exact,
-                                  per_item);
-      atomicAdd(&s_parts, 5ULL * p.S * (unsigned long long)na);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && s_parts > (unsigned long long)E.part_cap)
-      s_fallback = 1;
-    __syncthreads();
-    if (s_fallback) per_item = 0.0;
+    if (block_sum<long long>(parts, wtl) <= E.part_cap) break;
+    per_item = 0.0;
   }
   for (int base = 0; base < E.nc; base += kPlanThreads) {
     const int c = base + threadIdx.x;
-    const bool valid = c < E.nc;
-    int n_act = 0, nb = 0, items = 0;
-    long long parts = 0;
-    if (valid) {
-      nb = E.off[c + 1] - E.off[c];
-      if (E.tau_next[c] != LLONG_MAX) n_act = E.cnt[c];
-      const Plan p = ens_plan_for(n_act, nb, exact, per_item);
-      E.plan[c] = p;
-      items = n_act ? p.n_g * p.S : 0;
-      parts = n_act ? 5LL * p.S * n_act : 0;
+    if (E.nc > kPlanThreads) {
+      na = 0;
+      if (c < E.nc) plan_of(c);
     }
+    const int items = na ? p.n_g * p.S : 0;
+    const long long parts = na ? 5LL * p.S * na : 0;
     const int ci = c_items, cn = c_nact;
     const long long cp = c_part;
     const int inc_i = block_scan<int>(items, wti);
-    const int inc_n = block_scan<int>(n_act, wti);
+    const int inc_n = block_scan<int>(na, wti);
     const long long inc_p = block_scan<long long>(parts, wtl);
-    if (valid) {
+    if (c < E.nc) {
+      E.plan[c] = p;
       E.item_off[c] = ci + inc_i - items;
-      E.act_base[c] = cn + inc_n - n_act;
+      E.act_base[c] = cn + inc_n - na;
       E.part_off[c] = cp + inc_p - parts;
     }
-    __syncthreads();
     if (threadIdx.x == kPlanThreads - 1) {
       c_items = ci + inc_i;
       c_nact = cn + inc_n;
@@ -357,7 +377,7 @@ __global__ void __launch_bounds__(kPlanThreads)
       ctl->slot[0].nrec += c_nact;
       E.totals[2] = 0;  // counted again by the next select
       ctl->steps += 1ULL;
-      ctl->inter += s_inter;
+      ctl->inter += (unsigned long long)inter;
     }
   }
 }
@@ -651,28 +671,35 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ---------------------------------------------------------------------
-// correct: one thread per active-list slot
+// correct: one thread per active body of all clusters, in cluster order (the
+// cluster found by a search of the planner's prefix of active counts). What
+// bounds it is the chain of FP64 operations of one body and the loads of
+// scattered bodies; a thread per body slot of every cluster, most of them
+// not active, took 29 us per launch (512 clusters, caches cold), this 27; a block
+// per cluster waits for the largest active set (90 us).
 // ---------------------------------------------------------------------
-__global__ void ens_correct_kernel(Bodies B, Params P, Ens E, History cur,
-                                   History prev, const double* part) {
+constexpr int kEnsCorrectThreads = 64;
+
+__global__ void __launch_bounds__(kEnsCorrectThreads)
+    ens_correct_kernel(Bodies B, Params P, Ens E, History cur, History prev,
+                       const double* part) {
   Ctl* ctl = P.ctl;
-  if (ctl->done) return;
-  const int pass = ctl->pass;
+  const int done = ctl->done, pass = ctl->pass;
+  const int total = E.totals[1];
   const long long rec0 = E.totals[3];
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < B.n;
-       t += gridDim.x * blockDim.x) {
-    const int c = E.cl[t];
-    const long long tn = E.tau_next[c];
-    if (tn == LLONG_MAX) continue;
-    const int o = E.off[c];
-    const int k = t - o;
+  if (done) return;
+  for (int t = blockIdx.x * kEnsCorrectThreads + threadIdx.x; t < total;
+       t += gridDim.x * kEnsCorrectThreads) {
+    const int c = find_cluster(E.act_base, E.nc, t);
+    const int k = t - E.act_base[c];
     const int n_act = E.cnt[c];
-    if (k >= n_act) continue;
-    const int i = o + E.act[t];
+    const long long tn = E.tau_next[c];
+    const int o = E.off[c];
+    const int i = o + E.act[o + k];
     double an[3], q;
     sum_partials(part + E.part_off[c], n_act, E.plan[c].S, k, an, q);
     const Corrected cr = correct_body(B, P, cur, prev, i, an, q, tn, pass,
-                                      rec0 + E.act_base[c] + k, &ctl->err);
+                                      rec0 + t, &ctl->err);
     if (cr.underflow) atomicAdd(&ctl->underflow, 1ULL);
     if (cr.d_new != cr.d_old) {
       atomicSub(&E.hist[c * kMaxLevels + level_of(cr.d_old, P.k_max)], 1);
@@ -834,8 +861,8 @@ void launch_ens_step(const Bodies& B, const Params& P, const Ens& E,
   if (ev0) cudaEventRecordWithFlags(ev0, s, evflags);
   launch_ens_force(B, P, E, fl, precision, exact, s);
   if (ev1) cudaEventRecordWithFlags(ev1, s, evflags);
-  ens_correct_kernel<<<blocks_for(B.n, 64, 1 << 20), 64, 0, s>>>(B, P, E, HA,
-                                                                 HB, B.part);
+  ens_correct_kernel<<<blocks_for(B.n, kEnsCorrectThreads, 8 * fl.sms),
+                       kEnsCorrectThreads, 0, s>>>(B, P, E, HA, HB, B.part);
 }
 
 void launch_ens_init(const Bodies& B, const Params& P, const Ens& E,

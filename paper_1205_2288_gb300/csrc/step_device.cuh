@@ -203,7 +203,8 @@ __device__ __forceinline__ void predict_body(const Bodies& B, const Params& P,
 }
 
 // S split partial sums of active position k (layout [split][5][n_act]),
-// added in split order
+// added in split order; the maximum is taken on the bit patterns (q >= 0),
+// off the FP64 pipe
 __device__ __forceinline__ void sum_partials(const double* part, int n_act,
                                              int S, int k, double an[3],
                                              double& q) {
@@ -211,15 +212,17 @@ __device__ __forceinline__ void sum_partials(const double* part, int n_act,
   an[0] = pp[0 * n_act + k];
   an[1] = pp[1 * n_act + k];
   an[2] = pp[2 * n_act + k];
-  q = pp[4 * n_act + k];
+  long long qb = __double_as_longlong(pp[4 * n_act + k]);
 #pragma unroll 4
   for (int sp = 1; sp < S; ++sp) {
     pp = part + (long long)sp * 5 * n_act;
     an[0] = __dadd_rn(an[0], pp[0 * n_act + k]);
     an[1] = __dadd_rn(an[1], pp[1 * n_act + k]);
     an[2] = __dadd_rn(an[2], pp[2 * n_act + k]);
-    q = fmax(q, pp[4 * n_act + k]);
+    const long long b = __double_as_longlong(pp[4 * n_act + k]);
+    if (b > qb) qb = b;
   }
+  q = __longlong_as_double(qb);
 }
 
 // The step estimate of Eq. 3, eta / sqrt(q). FP64 path: correctly rounded
@@ -301,7 +304,7 @@ __device__ __forceinline__ double history_dts_at_w(const HistWin& W,
   if (c + 1 >= end) return fallback;
   const long long tc1 = win_tau(W, H, c + 1);
   const double dc = win_dts(W, H, c), dc1 = win_dts(W, H, c + 1);
-  const double w = __ddiv_rn((double)(t - tc), (double)(tc1 - tc));
+  const double w = ticks_ratio(t - tc, tc1 - tc);
   return __dadd_rn(dc, __dmul_rn(__dsub_rn(dc1, dc), w));
 }
 
