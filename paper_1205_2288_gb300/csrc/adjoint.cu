@@ -265,7 +265,7 @@ void replay_steps(tsbts_ctx* c, AdjCtx& A, long long s0, long long s1,
     }
     const long long T = A.tau[s];
     const int na = (int)(A.off[s + 1] - A.off[s]);
-    launch_step_force(c, A, A.act + A.off[s], na, A.plans[s], A.shapes[s].si);
+    launch_step_force(c, A, A.act + A.off[s], na, A.plans[s], A.shapes[s].sf);
     const bool more = s + 1 < s1;
     launch_adj_correct_predict(A.n, na, T, A.off[s], A.off[s + 1],
                                more ? A.tau[s + 1] : -1,
@@ -368,7 +368,7 @@ void enqueue_forward(tsbts_ctx* c, AdjCtx& A) {
   A.launches += 1;
   if (!st) {
     // the initial force, then the prediction to the first block time
-    launch_step_force(c, A, A.iota, A.n, A.plan_init, A.shape_init.si);
+    launch_step_force(c, A, A.iota, A.n, A.plan_init, A.shape_init.sf);
     launch_adj_init_accel(A.n, A.part, A.nsplit, fsum_of(A),
                           A.S > 0 ? A.tau[0] : -1, A.inv_ticks, A.mixed,
                           A.St, A.P, A.err, c->s);
@@ -820,7 +820,8 @@ int adjoint_init(tsbts_ctx* ctx, int64_t n, double eps, int64_t n_pass,
     A.plans.resize(A.S);
     long long cap_i = 0, cap_j = 0, grp_i = 0, grp_j = 0;
     auto need = [&](const VjpShape& v) {
-      cap_i = std::max(cap_i, (long long)v.si.groups * v.si.S * 4 * 128 /
+      cap_i = std::max(cap_i, (long long)v.si.groups *
+                                  std::max(v.si.S, v.sf.S) * 4 * 128 /
                                   v.si.tpt);
       cap_j = std::max(cap_j, (long long)v.sj.groups * v.sj.S * 4 * 128 /
                                   v.sj.tpt);

@@ -49,14 +49,11 @@ namespace {
 constexpr int kAdjThreads = 128;
 
 // tuning of the force vector-Jacobian product and the replay force
-// (compile-time; defaults measured on GB300): lanes per target, threads in
-// flight per SM that the split count aims at, most splits, sources per
-// shared-memory tile, unroll of the packed pair loop, register budget hint
+// (compile-time; defaults measured on GB300): lanes per target, most splits,
+// sources per shared-memory tile, unroll of the packed pair loop, register
+// budget hint
 #ifndef TSBTS_VJP_TPT
 #define TSBTS_VJP_TPT 4
-#endif
-#ifndef TSBTS_VJP_WANT
-#define TSBTS_VJP_WANT 512
 #endif
 #ifndef TSBTS_VJP_SMAX
 #define TSBTS_VJP_SMAX 16
@@ -65,14 +62,15 @@ constexpr int kAdjThreads = 128;
 #define TSBTS_VJP_TILE 512
 #endif
 #ifndef TSBTS_VJP_UNROLL
-#define TSBTS_VJP_UNROLL 2
+#define TSBTS_VJP_UNROLL 4
 #endif
 #ifndef TSBTS_VJP_MINB
 #define TSBTS_VJP_MINB 1
 #endif
 constexpr int kVjpTpt = TSBTS_VJP_TPT;
-constexpr int kVjpWant = TSBTS_VJP_WANT;
 constexpr int kVjpSmax = TSBTS_VJP_SMAX;
+constexpr int kVjpFewGroups = 8;  // target groups that take more splits
+constexpr int kVjpSmaxFew = 64;
 constexpr int kVjpMinBlocks = TSBTS_VJP_MINB;
 constexpr int kVjpUnroll = TSBTS_VJP_UNROLL;
 
@@ -626,10 +624,25 @@ struct VjpSm {
   double sums[4][kAdjThreads];
 };
 
-template <int kN>
-__device__ __forceinline__ void lane_reduce(double (&x)[kN], int tpt) {
-  for (int o = tpt >> 1; o > 0; o >>= 1)
-    for (int c = 0; c < kN; ++c) x[c] += __shfl_xor_sync(kFull, x[c], o);
+// Sums of the four components over the tpt lanes of a target, in a fixed
+// tree. From four lanes on, the first two exchanges split the components
+// between the lanes (a lane keeps two, then one), so the tree takes tpt / 2
+// + 1 FP64 additions per lane at tpt = 4 and one more per doubling instead
+// of four per level: an FP64 addition takes 64 cycles. Returns whether this
+// lane holds a final sum, in x[0], of component `comp`.
+__device__ __forceinline__ bool lane_reduce(double (&x)[4], int tpt, int lane,
+                                            int& comp) {
+  const int o1 = tpt >> 1, o2 = tpt >> 2;
+  const bool h1 = lane & o1, h2 = lane & o2;
+  double a = h1 ? x[2] : x[0], b = h1 ? x[3] : x[1];
+  a += __shfl_xor_sync(kFull, h1 ? x[0] : x[2], o1);
+  b += __shfl_xor_sync(kFull, h1 ? x[1] : x[3], o1);
+  double r = h2 ? b : a;
+  r += __shfl_xor_sync(kFull, h2 ? a : b, o2);
+  for (int o = tpt >> 3; o > 0; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+  comp = (h1 ? 2 : 0) + (h2 ? 1 : 0);
+  x[0] = r;
+  return (lane & (o2 - 1)) == 0;
 }
 
 struct VjpBlock {
@@ -679,37 +692,65 @@ __device__ __forceinline__ void vjp_finish(const VjpArgs& A, const VjpSide& V,
                                            const VjpBlock& B, int n_targets,
                                            double (&acc)[4], double* part,
                                            int* cnt, VjpSm& sm) {
-  lane_reduce(acc, V.tpt);
+  const int ig = kAdjThreads / V.tpt;
+  const bool spread = V.tpt >= 4;
+  int comp = 0;
+  bool holds = B.lane == 0;
+  if (spread)
+    holds = lane_reduce(acc, V.tpt, B.lane, comp);
+  else if (V.tpt == 2)
+    for (int c = 0; c < 4; ++c) acc[c] += __shfl_xor_sync(kFull, acc[c], 1);
   if (V.S == 1) {
-    if (B.live && B.lane == 0) vjp_store<kSide>(A, B.tgt, acc);
+    if (spread) {
+      // the four components back to the target's first lane
+      const int l0 = (threadIdx.x & 31) - B.lane;
+      double x[4];
+      for (int c = 0; c < 4; ++c)
+        x[c] = __shfl_sync(kFull, acc[0],
+                           l0 + (c >> 1) * (V.tpt >> 1) +
+                               (c & 1) * (V.tpt >> 2));
+      if (B.live && B.lane == 0) vjp_store<kSide>(A, B.tgt, x);
+    } else if (B.live && B.lane == 0) {
+      vjp_store<kSide>(A, B.tgt, acc);
+    }
     return;
   }
-  const int ig = kAdjThreads / V.tpt;
   double* gp = part + (long long)B.g * V.S * 4 * ig;
-  if (B.lane == 0)
-    for (int c = 0; c < 4; ++c) gp[((long long)B.sp * 4 + c) * ig + B.tl] = acc[c];
+  if (holds) {
+    double* q = gp + (long long)B.sp * 4 * ig + B.tl;
+    if (spread) {
+      q[comp * ig] = acc[0];
+    } else {
+      for (int c = 0; c < 4; ++c) q[c * ig] = acc[c];
+    }
+  }
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) sm.last = atomicAdd(&cnt[B.g], 1) == V.S - 1;
   __syncthreads();
   if (!sm.last) return;
   __threadfence();
-  for (int o = threadIdx.x; o < 4 * ig; o += kAdjThreads) {
-    const int c = o / ig, t = o - c * ig;
+  // each of the 4 ig sums over the splits by P neighbouring threads: thread
+  // r adds splits r, r + P, ..., eight loads in flight, then a fixed tree
+  const int P = spread ? min(V.tpt >> 2, 8) : 1;
+  for (int o = threadIdx.x; o < 4 * ig * P; o += kAdjThreads) {
+    const int r = o & (P - 1), v = o / P;
+    const int c = v / ig, t = v - c * ig;
     const double* q = gp + (long long)c * ig + t;
     const long long stride = 4LL * ig;
     double x = 0.0;
-    int sp = 0;
-    // eight loads in flight, then added in split order
-    for (; sp + 8 <= V.S; sp += 8) {
+    int sp = r;
+    for (; sp + 7 * P < V.S; sp += 8 * P) {
       double y[8];
 #pragma unroll
-      for (int w = 0; w < 8; ++w) y[w] = __ldcg(q + (sp + w) * stride);
+      for (int w = 0; w < 8; ++w) y[w] = __ldcg(q + (sp + w * P) * stride);
 #pragma unroll
       for (int w = 0; w < 8; ++w) x += y[w];
     }
-    for (; sp < V.S; ++sp) x += __ldcg(q + sp * stride);
-    sm.sums[c][t] = x;
+    for (; sp < V.S; sp += P) x += __ldcg(q + sp * stride);
+    // (4 ig P is a multiple of 32: whole warps are here)
+    for (int w = P >> 1; w > 0; w >>= 1) x += __shfl_xor_sync(kFull, x, w);
+    if (r == 0) sm.sums[c][t] = x;
   }
   __syncthreads();
   for (int t = threadIdx.x; t < ig; t += kAdjThreads) {
@@ -793,9 +834,13 @@ __device__ __forceinline__ void vjp_j_f64(const VjpArgs& A, int b, VjpSm& sm) {
 // arrays, and taken four at a time (128-bit shared loads) as two packed
 // pairs; every FMA-pipe operation works on two sources at once (f32x2).
 // A tile is padded to a multiple of 4 tpt with neutral sources (zero mass
-// or zero lam, far away), so every lane runs the same packed loop. A warp
-// whose target sits in the tile runs the masked loop, where the target's
-// own pair gets 1/s = 0 and adds exact zeros.
+// or zero lam, far away), so every lane runs the same packed loop. The warp
+// ORs the loop iterations that hold one of its targets; those (and all of
+// them where eps^2 is no normal float) run the masked form, where a target's
+// own pair gets 1/s = 0 and adds exact zeros, and the square root takes
+// subnormals; both forms round alike. (With every tile that holds a target
+// masked as a whole, a step on all bodies ran a quarter of its loops
+// masked.)
 constexpr int kVjpTile = TSBTS_VJP_TILE;
 constexpr float kFar = 1.0e18f;
 
@@ -830,7 +875,7 @@ __device__ __forceinline__ void pair_vjp_i2(const f2 (&ii)[9], f2 xh, f2 yh,
   const f2 s2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
   float s0, s1;
   upk(s2, s0, s1);
-  float r0 = rsqrtf(s0), r1 = rsqrtf(s1);
+  float r0 = rsqrt_of<kMask>(s0), r1 = rsqrt_of<kMask>(s1);
   if (kMask) {
     if (c == self) r0 = 0.f;
     if (c + 1 == self) r1 = 0.f;
@@ -860,7 +905,7 @@ __device__ __forceinline__ void pair_vjp_j2(const f2 (&jj)[6], f2 xh, f2 yh,
   const f2 s2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
   float s0, s1;
   upk(s2, s0, s1);
-  float r0 = rsqrtf(s0), r1 = rsqrtf(s1);
+  float r0 = rsqrt_of<kMask>(s0), r1 = rsqrt_of<kMask>(s1);
   if (kMask) {
     if (c == self) r0 = 0.f;
     if (c + 1 == self) r1 = 0.f;
@@ -882,6 +927,21 @@ __device__ __forceinline__ float hsum(f2 x) {
   return a + b;
 }
 
+// the iterations (one quad per lane each) of a tile's pair loop that hold
+// the own source sc (tile slot, < 0: none) of a target of this warp; at
+// most kVjpTile / 4 = 128 iterations, whose numbers are taken modulo 64 (the
+// loop rotates the mask; a masked iteration that needs none is only slower)
+__device__ __forceinline__ unsigned long long self_mask(int sc, int step,
+                                                        bool normal) {
+  if (!normal) return ~0ULL;
+  const int own = sc < 0 ? -1 : sc / step & 63;
+  const unsigned lo =
+      __reduce_or_sync(kFull, own >= 0 && own < 32 ? 1u << own : 0u);
+  const unsigned hi =
+      __reduce_or_sync(kFull, own >= 32 ? 1u << (own - 32) : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+
 __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
                                             VjpSmem& T0, VjpSm& sm) {
   const VjpSide& V = A.V.si;
@@ -897,11 +957,12 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
                     pk(lm.x, lm.x), pk(lm.y, lm.y), pk(lm.z, lm.z)};
   const f2 e2 = pk(A.eps2f, A.eps2f);
   const int step = 4 * V.tpt;
+  const bool normal = normal_eps2(A.eps2f);
   DS dacc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};  // W, U
   VjpTileI& T = T0.i;
   for (int jt = B.beg; jt < B.end; jt += kVjpTile) {
     const int cnt = min(kVjpTile, B.end - jt);
-    const int cntp = (cnt + step - 1) / step * step;
+    const int iters = (cnt + step - 1) / step, cntp = iters * step;
     __syncthreads();
     for (int c = threadIdx.x; c < cntp; c += kAdjThreads) {
       if (c < cnt) {
@@ -917,28 +978,36 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
     const bool self_here = B.live && bi >= jt && bi < jt + cnt;
     const int sc = self_here ? bi - jt : -1;
     f2 W = pk(0.f, 0.f), Ux = W, Uy = W, Uz = W;
-    if (__any_sync(kFull, self_here)) {
-      for (int c = 4 * B.lane; c < cntp; c += step) {
-        const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
-                         zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
-                         xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
-                         zl = ld4(&T.zl[c]);
-        pair_vjp_i2<true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
-                          e2, W, Ux, Uy, Uz);
-        pair_vjp_i2<true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
-                          sc, e2, W, Ux, Uy, Uz);
-      }
-    } else {
-#pragma unroll kVjpUnroll
-      for (int c = 4 * B.lane; c < cntp; c += step) {
-        const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
-                         zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
-                         xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
-                         zl = ld4(&T.zl[c]);
-        pair_vjp_i2<false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c,
-                           -1, e2, W, Ux, Uy, Uz);
-        pair_vjp_i2<false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
-                           -1, e2, W, Ux, Uy, Uz);
+    unsigned long long mask = self_mask(sc, step, normal);
+    int c = 4 * B.lane;
+    // (cntp is a whole number of steps; two to an unrolled iteration)
+    for (int m = 0; m < iters; m += kVjpUnroll,
+             mask = (mask >> kVjpUnroll) | (mask << (64 - kVjpUnroll))) {
+      if (m + kVjpUnroll <= iters &&
+          (mask & ((1ULL << kVjpUnroll) - 1)) == 0) {
+#pragma unroll
+        for (int w = 0; w < kVjpUnroll; ++w, c += step) {
+          const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
+                           zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
+                           xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
+                           zl = ld4(&T.zl[c]);
+          pair_vjp_i2<false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c,
+                             -1, e2, W, Ux, Uy, Uz);
+          pair_vjp_i2<false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+                             -1, e2, W, Ux, Uy, Uz);
+        }
+      } else {
+#pragma unroll 1
+        for (int w = 0; w < kVjpUnroll && m + w < iters; ++w, c += step) {
+          const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
+                           zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
+                           xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
+                           zl = ld4(&T.zl[c]);
+          pair_vjp_i2<true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
+                            e2, W, Ux, Uy, Uz);
+          pair_vjp_i2<true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+                            sc, e2, W, Ux, Uy, Uz);
+        }
       }
     }
     ds_add(dacc[0], hsum(W));
@@ -947,7 +1016,7 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
     ds_add(dacc[3], hsum(Uz));
   }
   double acc[4];
-  for (int c = 0; c < 4; ++c) acc[c] = (double)dacc[c].hi + (double)dacc[c].lo;
+  for (int c = 0; c < 4; ++c) acc[c] = to_double(dacc[c]);
   vjp_finish<0>(A, V, B, A.n_act, acc, A.O.part_i, A.O.cnt_i, sm);
 }
 
@@ -965,11 +1034,12 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
   const f2 e2 = pk(A.eps2f, A.eps2f);
   const f2 m3 = pk(-3.f, -3.f);
   const int step = 4 * V.tpt;
+  const bool normal = normal_eps2(A.eps2f);
   DS dacc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};  // G, Z
   VjpTileJ& T = T0.j;
   for (int kt = B.beg; kt < B.end; kt += kVjpTile) {
     const int cnt = min(kVjpTile, B.end - kt);
-    const int cntp = (cnt + step - 1) / step * step;
+    const int iters = (cnt + step - 1) / step, cntp = iters * step;
     __syncthreads();
     for (int c = threadIdx.x; c < cntp; c += kAdjThreads) {
       if (c < cnt) {
@@ -988,30 +1058,38 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
     const bool self_here = sj >= kt && sj < kt + cnt;
     const int sc = self_here ? sj - kt : -1;
     f2 G0 = pk(0.f, 0.f), G1 = G0, G2 = G0, Z = G0;
-    if (__any_sync(kFull, self_here)) {
-      for (int c = 4 * B.lane; c < cntp; c += step) {
-        const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
-                         zh = ld4(&T.zh[c]), xl = ld4(&T.xl[c]),
-                         yl = ld4(&T.yl[c]), zl = ld4(&T.zl[c]),
-                         lx = ld4(&T.lx[c]), ly = ld4(&T.ly[c]),
-                         lz = ld4(&T.lz[c]);
-        pair_vjp_j2<true>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x, ly.x,
-                          lz.x, c, sc, e2, m3, G0, G1, G2, Z);
-        pair_vjp_j2<true>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y, ly.y,
-                          lz.y, c + 2, sc, e2, m3, G0, G1, G2, Z);
-      }
-    } else {
-#pragma unroll kVjpUnroll
-      for (int c = 4 * B.lane; c < cntp; c += step) {
-        const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
-                         zh = ld4(&T.zh[c]), xl = ld4(&T.xl[c]),
-                         yl = ld4(&T.yl[c]), zl = ld4(&T.zl[c]),
-                         lx = ld4(&T.lx[c]), ly = ld4(&T.ly[c]),
-                         lz = ld4(&T.lz[c]);
-        pair_vjp_j2<false>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x,
-                           ly.x, lz.x, c, -1, e2, m3, G0, G1, G2, Z);
-        pair_vjp_j2<false>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y,
-                           ly.y, lz.y, c + 2, -1, e2, m3, G0, G1, G2, Z);
+    unsigned long long mask = self_mask(sc, step, normal);
+    int c = 4 * B.lane;
+    // (cntp is a whole number of steps; two to an unrolled iteration)
+    for (int m = 0; m < iters; m += kVjpUnroll,
+             mask = (mask >> kVjpUnroll) | (mask << (64 - kVjpUnroll))) {
+      if (m + kVjpUnroll <= iters &&
+          (mask & ((1ULL << kVjpUnroll) - 1)) == 0) {
+#pragma unroll
+        for (int w = 0; w < kVjpUnroll; ++w, c += step) {
+          const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
+                           zh = ld4(&T.zh[c]), xl = ld4(&T.xl[c]),
+                           yl = ld4(&T.yl[c]), zl = ld4(&T.zl[c]),
+                           lx = ld4(&T.lx[c]), ly = ld4(&T.ly[c]),
+                           lz = ld4(&T.lz[c]);
+          pair_vjp_j2<false>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x,
+                             ly.x, lz.x, c, -1, e2, m3, G0, G1, G2, Z);
+          pair_vjp_j2<false>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y,
+                             ly.y, lz.y, c + 2, -1, e2, m3, G0, G1, G2, Z);
+        }
+      } else {
+#pragma unroll 1
+        for (int w = 0; w < kVjpUnroll && m + w < iters; ++w, c += step) {
+          const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
+                           zh = ld4(&T.zh[c]), xl = ld4(&T.xl[c]),
+                           yl = ld4(&T.yl[c]), zl = ld4(&T.zl[c]),
+                           lx = ld4(&T.lx[c]), ly = ld4(&T.ly[c]),
+                           lz = ld4(&T.lz[c]);
+          pair_vjp_j2<true>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x, ly.x,
+                            lz.x, c, sc, e2, m3, G0, G1, G2, Z);
+          pair_vjp_j2<true>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y, ly.y,
+                            lz.y, c + 2, sc, e2, m3, G0, G1, G2, Z);
+        }
       }
     }
     ds_add(dacc[0], hsum(G0));
@@ -1020,7 +1098,7 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
     ds_add(dacc[3], hsum(Z));
   }
   double acc[4];
-  for (int c = 0; c < 4; ++c) acc[c] = (double)dacc[c].hi + (double)dacc[c].lo;
+  for (int c = 0; c < 4; ++c) acc[c] = to_double(dacc[c]);
   vjp_finish<1>(A, V, B, A.n, acc, A.O.part_j, A.O.cnt_j, sm);
 }
 
@@ -1038,7 +1116,7 @@ __device__ __forceinline__ void pair_force2(const f2 (&ii)[6], f2 xh, f2 yh,
   const f2 s2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
   float s0, s1;
   upk(s2, s0, s1);
-  float r0 = rsqrtf(s0), r1 = rsqrtf(s1);
+  float r0 = rsqrt_of<kMask>(s0), r1 = rsqrt_of<kMask>(s1);
   if (kMask) {
     if (c == self) r0 = 0.f;
     if (c + 1 == self) r1 = 0.f;
@@ -1062,11 +1140,12 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
                     pk(il.x, il.x), pk(il.y, il.y), pk(il.z, il.z)};
   const f2 e2 = pk(A.eps2f, A.eps2f);
   const int step = 4 * V.tpt;
+  const bool normal = normal_eps2(A.eps2f);
   DS dacc[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   VjpTileI& T = T0.i;
   for (int jt = B.beg; jt < B.end; jt += kVjpTile) {
     const int cnt = min(kVjpTile, B.end - jt);
-    const int cntp = (cnt + step - 1) / step * step;
+    const int iters = (cnt + step - 1) / step, cntp = iters * step;
     __syncthreads();
     for (int c = threadIdx.x; c < cntp; c += kAdjThreads) {
       if (c < cnt) {
@@ -1082,28 +1161,36 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
     const bool self_here = B.live && bi >= jt && bi < jt + cnt;
     const int sc = self_here ? bi - jt : -1;
     f2 ax = pk(0.f, 0.f), ay = ax, az = ax;
-    if (__any_sync(kFull, self_here)) {
-      for (int c = 4 * B.lane; c < cntp; c += step) {
-        const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
-                         zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
-                         xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
-                         zl = ld4(&T.zl[c]);
-        pair_force2<true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
-                          e2, ax, ay, az);
-        pair_force2<true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
-                          sc, e2, ax, ay, az);
-      }
-    } else {
-#pragma unroll kVjpUnroll
-      for (int c = 4 * B.lane; c < cntp; c += step) {
-        const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
-                         zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
-                         xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
-                         zl = ld4(&T.zl[c]);
-        pair_force2<false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, -1,
-                           e2, ax, ay, az);
-        pair_force2<false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
-                           -1, e2, ax, ay, az);
+    unsigned long long mask = self_mask(sc, step, normal);
+    int c = 4 * B.lane;
+    // (cntp is a whole number of steps; two to an unrolled iteration)
+    for (int m = 0; m < iters; m += kVjpUnroll,
+             mask = (mask >> kVjpUnroll) | (mask << (64 - kVjpUnroll))) {
+      if (m + kVjpUnroll <= iters &&
+          (mask & ((1ULL << kVjpUnroll) - 1)) == 0) {
+#pragma unroll
+        for (int w = 0; w < kVjpUnroll; ++w, c += step) {
+          const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
+                           zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
+                           xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
+                           zl = ld4(&T.zl[c]);
+          pair_force2<false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, -1,
+                             e2, ax, ay, az);
+          pair_force2<false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+                             -1, e2, ax, ay, az);
+        }
+      } else {
+#pragma unroll 1
+        for (int w = 0; w < kVjpUnroll && m + w < iters; ++w, c += step) {
+          const ulonglong2 xh = ld4(&T.xh[c]), yh = ld4(&T.yh[c]),
+                           zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
+                           xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
+                           zl = ld4(&T.zl[c]);
+          pair_force2<true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
+                            e2, ax, ay, az);
+          pair_force2<true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+                            sc, e2, ax, ay, az);
+        }
       }
     }
     ds_add(dacc[0], hsum(ax));
@@ -1111,7 +1198,7 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
     ds_add(dacc[2], hsum(az));
   }
   double acc[4];
-  for (int c = 0; c < 3; ++c) acc[c] = (double)dacc[c].hi + (double)dacc[c].lo;
+  for (int c = 0; c < 3; ++c) acc[c] = to_double(dacc[c]);
   acc[3] = 0.0;
   vjp_finish<2>(A, V, B, A.n_act, acc, A.O.part_i, A.O.cnt_i, sm);
 }
@@ -1222,39 +1309,96 @@ int body_grid(int n) {
   return std::max(1, std::min((n + kBodyThreads - 1) / kBodyThreads, 16384));
 }
 
-// Both sides: kVjpTpt lanes per target (more, up to 32, when the targets
-// are few; fewer when the sources are few), 128 / tpt targets per block
-// sharing each source tile, and as many source
-// splits (at most kVjpSmax, each lane at least 16 sources) as fill about
-// kVjpWant threads per SM.
-VjpSide choose_side(long long nt, long long ns, int sms) {
-  const long long want = (long long)sms * kVjpWant;
+// Lanes per target of one side of the product: kVjpTpt (more, up to 32, when
+// the targets are few; fewer when the sources are few); 128 / tpt targets
+// per block share each source tile.
+VjpSide side_of(long long nt, long long ns) {
+  VjpSide v{};
   int tpt = kVjpTpt;
   // few targets: more lanes each, so that the block's threads are used
   while (tpt < 32 && (kAdjThreads / (2 * tpt)) >= nt) tpt *= 2;
   while (tpt > 1 && ns < 16LL * tpt) tpt >>= 1;
   const int ig = kAdjThreads / tpt;
-  VjpSide v{};
-  const long long groups = std::max<long long>(1, (nt + ig - 1) / ig);
-  long long S = (want + groups * kAdjThreads - 1) / (groups * kAdjThreads);
-  S = std::min<long long>(S, kVjpSmax);
-  S = std::min<long long>(S, std::max<long long>(1, ns / (16LL * tpt)));
-  S = std::max<long long>(S, 1);
-  long long chunk = std::max<long long>(1, (ns + S - 1) / S);
-  S = std::max<long long>(1, (ns + chunk - 1) / chunk);
   v.tpt = tpt;
-  v.S = (int)S;
-  v.chunk = (int)chunk;
-  v.groups = (int)groups;
+  v.groups = (int)std::max<long long>(1, (nt + ig - 1) / ig);
   return v;
+}
+
+// one side's source splits set to S (fewer where chunks would be empty)
+void set_splits(VjpSide& v, long long ns, long long S) {
+  const long long chunk = std::max<long long>(1, (ns + S - 1) / S);
+  v.chunk = (int)chunk;
+  v.S = (int)std::max<long long>(1, (ns + chunk - 1) / chunk);
+}
+
+// split counts a side may take: at least one quad per lane for few target
+// groups, else 16 sources per lane
+int split_choices(const VjpSide& v, long long ns, int (&out)[17]) {
+  static const int kS[17] = {1,  2,  3,  4,  5,  6,  7,  8, 10,
+                             12, 14, 16, 20, 24, 32, 48, 64};
+  const bool few = v.groups <= kVjpFewGroups;
+  const long long cap = std::min<long long>(
+      few ? kVjpSmaxFew : kVjpSmax, ns / ((few ? 4LL : 16LL) * v.tpt));
+  int m = 0;
+  for (int S : kS)
+    if (S == 1 || S <= cap) out[m++] = S;
+  return m;
+}
+
+// Split counts of the launch's sides (si alone, or both) with the least
+// estimated time, in sources per lane: the SM with the most blocks runs its
+// share at full rate with kVjpResident of them, one block alone at about
+// half that, and each block adds kVjpBlockCost (bodies loaded, a tile
+// staged, sums over lanes and splits). Splits fixed by a number of threads
+// per SM for each side by itself left 1536 blocks of a step on all 8192
+// bodies on 608 places, the last of three waves half empty.
+constexpr int kVjpResident = 4;
+constexpr double kVjpBlockCost = 32.0;
+
+void choose_splits(VjpSide& si, long long ns_i, VjpSide* sj, long long ns_j,
+                   int sms) {
+  int ci[17], cj[17] = {1};
+  const int mi = split_choices(si, ns_i, ci);
+  const int mj = sj ? split_choices(*sj, ns_j, cj) : 1;
+  double best = 1e300;
+  int bi = 1, bj = 1;
+  for (int x = 0; x < mi; ++x)
+    for (int y = 0; y < mj; ++y) {
+      const double wi =
+          (double)((ns_i + ci[x] - 1) / ci[x] + si.tpt - 1) / si.tpt;
+      double blocks = (double)si.groups * ci[x];
+      double work = blocks * (wi + kVjpBlockCost), longest = wi;
+      if (sj) {
+        const double wj =
+            (double)((ns_j + cj[y] - 1) / cj[y] + sj->tpt - 1) / sj->tpt;
+        const double b = (double)sj->groups * cj[y];
+        work += b * (wj + kVjpBlockCost);
+        blocks += b;
+        longest = std::max(longest, wj);
+      }
+      const double per_sm = (double)(long long)((blocks + sms - 1) / sms);
+      const double t = std::max(0.5 * (longest + kVjpBlockCost),
+                                work / blocks * per_sm / kVjpResident);
+      // (near-ties go to fewer splits)
+      if (t + 0.005 * (ci[x] + cj[y]) < best) {
+        best = t + 0.005 * (ci[x] + cj[y]);
+        bi = ci[x];
+        bj = cj[y];
+      }
+    }
+  set_splits(si, ns_i, bi);
+  if (sj) set_splits(*sj, ns_j, bj);
 }
 
 }  // namespace
 
 VjpShape vjp_shape(int n, int n_act, int sms) {
   VjpShape s;
-  s.si = choose_side(n_act, n, sms);
-  s.sj = choose_side(n, n_act, sms);
+  s.si = side_of(n_act, n);
+  s.sf = s.si;
+  s.sj = side_of(n, n_act);
+  choose_splits(s.si, n, &s.sj, n_act, sms);
+  choose_splits(s.sf, n, nullptr, 0, sms);
   return s;
 }
 

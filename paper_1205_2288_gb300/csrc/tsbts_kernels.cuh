@@ -121,9 +121,10 @@ struct VjpSide {
   int tpt, S, chunk, groups;
 };
 // i side: targets are the active bodies, sources every body; j side:
-// targets every body, sources the active bodies
+// targets every body, sources the active bodies; sf: the i side's split of
+// a replay force launch, which runs without a j side
 struct VjpShape {
-  VjpSide si, sj;
+  VjpSide si, sj, sf;
 };
 VjpShape vjp_shape(int n, int n_act, int sms);
 // results of one force vector-Jacobian product: u[3] per active slot (i
