@@ -117,6 +117,7 @@ ForceArgs force_args_engine(tsbts_ctx* c, int p) {
   fa.eps2 = c->eps * c->eps;
   fa.eps2f = (float)(c->eps * c->eps);
   fa.exact = c->exact;
+  fa.no_phi = 1;
   return fa;
 }
 
@@ -161,10 +162,19 @@ void enqueue_step(tsbts_ctx* c, int p, int ev_slot, bool capturing) {
   }
   ck(launch_select_predict(c->B, c->P, HA, HB, p, false, c->s),
      "select/predict launch");
+  ForceArgs fa = force_args_engine(c, p);
+  if (c->B.order) {
+    // spatial order: the j records and the active list are by slot
+    fa.idx = c->B.aslot;
+    fa.meta = c->B.meta;
+    fa.far_min = c->n / kFarMinShare;
+    fa.amask = c->B.amask;
+    fa.order = c->B.order;
+    fa.act = c->B.act;
+  }
   if (ev_slot >= 0)
     ck(cudaEventRecordWithFlags(c->ev[2 * ev_slot], c->s, evflags), "event");
-  ck(launch_force(c->cfg.precision, force_args_engine(c, p), c->fl, c->s,
-                  &c->pt, false),
+  ck(launch_force(c->cfg.precision, fa, c->fl, c->s, &c->pt, false),
      "force launch");
   if (ev_slot >= 0)
     ck(cudaEventRecordWithFlags(c->ev[2 * ev_slot + 1], c->s, evflags),
@@ -341,6 +351,14 @@ int step_era_impl(tsbts_ctx* c, long long tau_end) {
         own_eras ? tau_end : std::min(c->t_sys + era_ticks(c), tau_end);
     launch_copy_state(c->snap, c->B, c->s);
     c->launches += 1;
+    if (c->B.order) {
+      // the bodies' spatial order at the era start serves its passes
+      c->launches += launch_spatial_order(c->n, c->B.r[0], c->B.r[1],
+                                          c->B.r[2], 1, c->d_sort,
+                                          c->sort_key, c->B.order, nullptr,
+                                          c->s);
+      ck(cudaGetLastError(), "spatial order");
+    }
     // counters at the era start: an era re-run after the history grew
     // counts (and logs) only the run that is kept
     read_ctl(c);
@@ -444,7 +462,7 @@ int step_era_impl(tsbts_ctx* c, long long tau_end) {
   return TSBTS_OK;
 }
 
-void setup_bodies(tsbts_ctx* c, int n) {
+void setup_bodies(tsbts_ctx* c, int n, bool sorted) {
   Bodies& B = c->B;
   B = Bodies{};
   B.n = n;
@@ -476,6 +494,15 @@ void setup_bodies(tsbts_ctx* c, int n) {
   B.seg = dalloc<double>(L, 18 * (size_t)n);
   B.part_cap = force_partial_capacity(c->fl, n);
   B.part = dalloc<double>(L, B.part_cap);
+  if (sorted) {
+    const size_t words = (size_t)(n + 31) / 32;
+    B.order = dalloc<int>(L, n);
+    B.aslot = dalloc<int>(L, n);
+    B.amask = dalloc<unsigned>(L, words);
+    B.meta = dalloc<float4>(L, 2 * words);
+    c->sort_key = dalloc<unsigned long long>(L, sort_capacity(n));
+    c->d_sort = dalloc<double>(L, 128);
+  }
   Bodies& S = c->snap;
   S = Bodies{};
   S.n = n;
@@ -617,7 +644,10 @@ int init_common(tsbts_ctx* c, int64_t n, const double* m, const double* r,
     c->correct_grid = std::max(1, std::min(c->sms * 32, (c->n + 31) / 32));
     c->ensemble = false;
     c->nc = 0;
-    setup_bodies(c, (int)n);
+    // large mixed systems keep their j records in spatial order
+    setup_bodies(c, (int)n,
+                 c->cfg.precision == TSBTS_MIXED && !ens &&
+                     n >= kSortMinBodies && n <= kSortMaxBodies);
     if (ens) {
       c->pt = PlanTable{};
       setup_ensemble(c, *ens);
@@ -720,7 +750,38 @@ struct Scratch {
   double* part = nullptr;
   int* nsplit = nullptr;
   int* iota = nullptr;    // 0, 1, ..., n_cap - 1 (active list for tuning)
+  // spatial order (calls that sort): order, slot, list and pos in `sort_i`
+  // (4 n_cap), keys, subtile summaries, 128 doubles
+  int* sort_i = nullptr;
+  unsigned long long* key = nullptr;
+  float4* meta = nullptr;
+  double* scale = nullptr;
+  int sort_cap = 0;       // bodies (and active bodies) it has room for
 };
+
+void free_sort(Scratch& S) {
+  cudaFree(S.sort_i);
+  cudaFree(S.key);
+  cudaFree(S.meta);
+  cudaFree(S.scale);
+  S.sort_i = nullptr;
+  S.key = nullptr;
+  S.meta = nullptr;
+  S.scale = nullptr;
+  S.sort_cap = 0;
+}
+
+// Whether a mixed force call sorts its bodies: the sorts of the bodies and of
+// the active list take about 0.2 ms together, what far pairs save is about
+// a third of the time (2^31 interactions: 1.9 ms), and the active bodies
+// have to be dense enough for 256 of them to fill a small box.
+bool force_sorts(int precision, int64_t n, int64_t n_act, double eps) {
+  const float eps2 = (float)(eps * eps);
+  return precision == TSBTS_MIXED && n >= kSortMinBodies &&
+         n <= kSortMaxBodies && n_act >= n / kFarMinShare &&
+         n_act <= kSortMaxBodies && n * n_act >= (1LL << 31) &&
+         eps2 >= 1.17549435e-38f;
+}
 std::mutex g_scratch_mu;
 std::vector<Scratch> g_scratch;
 
@@ -1184,6 +1245,7 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
       cudaFree(S.part);
       cudaFree(S.nsplit);
       cudaFree(S.iota);
+      free_sort(S);
       S = Scratch{};
       const int ncap = (int)std::max<int64_t>(n, S.n_cap);
       ck(cudaMalloc(&S.soa, sizeof(double) * 7 * (size_t)ncap), "scratch");
@@ -1202,10 +1264,36 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
     const int ni = (int)n;
     double* x = S.soa;
     float4* j4 = S.j4;
-    ck(launch_pack_aos(precision, ni, m, r, v, x, x + ni, x + 2LL * ni,
-                       x + 3LL * ni, x + 4LL * ni, x + 5LL * ni, x + 6LL * ni,
-                       j4, j4 + ni, j4 + 2LL * ni, s),
-       "pack");
+    const bool sorts = force_sorts(precision, n, n_act, eps);
+    if (sorts) {
+      const int need = (int)std::max(n, n_act);
+      if (S.sort_cap < need) {
+        ck(cudaDeviceSynchronize(), "synchronize before scratch growth");
+        free_sort(S);
+        ck(cudaMalloc(&S.sort_i, sizeof(int) * 4 * (size_t)need), "scratch");
+        ck(cudaMalloc(&S.key, sizeof(unsigned long long) *
+                                  (size_t)sort_capacity(need)),
+           "scratch");
+        ck(cudaMalloc(&S.meta, sizeof(float4) * 2 * ((size_t)need / 32 + 1)),
+           "scratch");
+        ck(cudaMalloc(&S.scale, sizeof(double) * 128), "scratch");
+        S.sort_cap = need;
+      }
+      int* order = S.sort_i;
+      int* slot = order + S.sort_cap;
+      launch_spatial_order(ni, r, r + 1, r + 2, 3, S.scale, S.key, order,
+                           slot, s);
+      launch_sorted_list((int)n_act, idx, slot, S.key, slot + S.sort_cap,
+                         slot + 2LL * S.sort_cap, s);
+      ck(launch_pack_sorted(ni, order, m, r, v, j4, j4 + ni, j4 + 2LL * ni,
+                            S.meta, s),
+         "pack");
+    } else {
+      ck(launch_pack_aos(precision, ni, m, r, v, x, x + ni, x + 2LL * ni,
+                         x + 3LL * ni, x + 4LL * ni, x + 5LL * ni,
+                         x + 6LL * ni, j4, j4 + ni, j4 + 2LL * ni, s),
+         "pack");
+    }
     ForceArgs fa{};
     fa.n = ni;
     fa.m = x + 6LL * ni;
@@ -1227,7 +1315,12 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
                (exact_order == 1 || (exact_order < 0 && n <= 8192));
     fa.plan = plan_force(precision, fa.exact, (int)n_act, ni, fl,
                          S.part_cap);
-    if (precision == TSBTS_MIXED && ni <= (1 << 20)) {
+    if (sorts) {
+      fa.idx = S.sort_i + 2LL * S.sort_cap;
+      fa.meta = S.meta;
+      fa.far_min = 0;
+      fa.plan.S = far_splits_host((int)n_act, ni, fl.grid, S.part_cap);
+    } else if (precision == TSBTS_MIXED && ni <= (1 << 20)) {
       // measured plans: the first call for a new n tunes them on these j
       // records and caches the table for the process
       const std::vector<Plan>* tp = tuned_plans(dev, ni, fl.grid);
@@ -1251,8 +1344,9 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
                    fa.plan.n_g, fa.plan.S, fa.plan.chunk,
                    fa.plan.direct ? "direct" : "tiled");
     ck(launch_force(precision, fa, fl, s), "force");
-    ck(launch_force_finalize(S.part, fa.exact ? 1 : fa.plan.S, (int)n_act, a,
-                             phi, q, s),
+    ck(launch_force_finalize(S.part, fa.exact ? 1 : fa.plan.S, (int)n_act,
+                             sorts ? S.sort_i + 3LL * S.sort_cap : nullptr,
+                             a, phi, q, s),
        "force finalize");
     return TSBTS_OK;
   } catch (const CudaFail& f) {
@@ -1274,6 +1368,7 @@ int tsbts_release_scratch(void) {
   cudaFree(S.part);
   cudaFree(S.nsplit);
   cudaFree(S.iota);
+  free_sort(S);
   S = Scratch{};
   return TSBTS_OK;
 }
@@ -1409,8 +1504,8 @@ extern "C" int tsbts_force_static(int precision, int exact_order, int64_t n,
   fa.has_plan = 1;
   e = launch_force(precision, fa, fl, s);
   if (e != cudaSuccess) return failed("force", e);
-  e = launch_force_finalize(part, fa.exact ? 1 : fa.plan.S, (int)n_act, a,
-                            phi, q, s);
+  e = launch_force_finalize(part, fa.exact ? 1 : fa.plan.S, (int)n_act,
+                            nullptr, a, phi, q, s);
   if (e != cudaSuccess) return failed("force finalize", e);
   return TSBTS_OK;
 }

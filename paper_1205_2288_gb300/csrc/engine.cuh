@@ -53,6 +53,8 @@ struct tsbts_ctx {
   Ctl* h_ctl = nullptr;  // pinned mirror
   double* d_w = nullptr;
   double* d_eout = nullptr;
+  unsigned long long* sort_key = nullptr;  // spatial order (large systems)
+  double* d_sort = nullptr;
   int* d_nsplit = nullptr;  // scratch for init's split count
   PlanTable pt{};            // force work plan per bucket of active counts
   ForceLaunch fl{};

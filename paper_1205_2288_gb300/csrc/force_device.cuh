@@ -87,6 +87,7 @@ __device__ __forceinline__ Plan tiled_plan_warp(int n_act, int n, int grid,
   return p;
 }
 
+template <bool kPhi = true>
 __device__ __forceinline__ void write_partial(const ForceArgs& A, int n_act,
                                               int split, int k, double ax,
                                               double ay, double az, double ph,
@@ -98,7 +99,7 @@ __device__ __forceinline__ void write_partial(const ForceArgs& A, int n_act,
   p[0 * n_act + k] = ax;
   p[1 * n_act + k] = ay;
   p[2 * n_act + k] = az;
-  p[3 * n_act + k] = ph;
+  if (kPhi) p[3 * n_act + k] = ph;
   p[4 * n_act + k] = q;
 }
 
@@ -543,6 +544,10 @@ struct J2 {
   f2 xh, yh, zh, m, xl, yl, zl, u, v, w;
 };
 
+__device__ __forceinline__ ulonglong2 lds4(const float* p) {
+  return *reinterpret_cast<const ulonglong2*>(p);
+}
+
 // j = t .. t + 3 (t a multiple of 4): one 128-bit shared load per component
 template <int TJ>
 __device__ __forceinline__ void load_j4(const MixTile<TJ>& T, int t, J2& a,
@@ -575,7 +580,7 @@ __device__ __forceinline__ bool normal_eps2(float eps2) {
 // kSafe: any s^2 >= 0 (rsqrtf), and the pair with tile index `self` is the
 // body itself: its 1/s is set to 0, so it adds exact zeros and the sums
 // equal those of the loop over the other j.
-template <bool kSafe>
+template <bool kPhi, bool kSafe, bool kCrit = true>
 __device__ __forceinline__ void pair_mixed2(const f2 (&ii)[9], const J2& J,
                                             int t, f2 eps2, f2 (&s)[4],
                                             float& q, int self = -1) {
@@ -597,16 +602,18 @@ __device__ __forceinline__ void pair_mixed2(const f2 (&ii)[9], const J2& J,
   s[0] = fma2(mr3, dx, s[0]);
   s[1] = fma2(mr3, dy, s[1]);
   s[2] = fma2(mr3, dz, s[2]);
-  s[3] = add2(s[3], mr);
-  const f2 wx = sub2(J.u, ii[6]);
-  const f2 wy = sub2(J.v, ii[7]);
-  const f2 wz = sub2(J.w, ii[8]);
-  const f2 w2 = fma2(wx, wx, fma2(wy, wy, mul2(wz, wz)));
-  const f2 c = mul2(w2, rinv2);
-  float c0, c1, m0, m1;
-  upk(c, c0, c1);
-  upk(mr3, m0, m1);
-  q = max3(max3(q, c0, m0), c1, m1);
+  if (kPhi) s[3] = add2(s[3], mr);
+  if (kCrit) {
+    const f2 wx = sub2(J.u, ii[6]);
+    const f2 wy = sub2(J.v, ii[7]);
+    const f2 wz = sub2(J.w, ii[8]);
+    const f2 w2 = fma2(wx, wx, fma2(wy, wy, mul2(wz, wz)));
+    const f2 c = mul2(w2, rinv2);
+    float c0, c1, m0, m1;
+    upk(c, c0, c1);
+    upk(mr3, m0, m1);
+    q = max3(max3(q, c0, m0), c1, m1);
+  }
 }
 
 // x as a double, by moving its exponent and significand (the FP64 pipe,
@@ -633,7 +640,7 @@ __device__ __forceinline__ double to_double(DS a) {
 // only those iterations (and all of them where eps^2 is no normal float)
 // run the masked form. Both forms round alike, so a body's sums do not
 // depend on its warp-mates.
-template <int JG>
+template <int JG, bool kPhi>
 __device__ __forceinline__ void mixed_item(const ForceArgs& A, int n_act,
                                            const Plan& P, int g, int split,
                                            MixTile<kTileMix>& T) {
@@ -716,8 +723,8 @@ __device__ __forceinline__ void mixed_item(const ForceArgs& A, int n_act,
             load_j4(T, c0 + 4 * JG * u, a, b);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-              pair_mixed2<false>(ii[r], a, 0, e2, p[r], q[r]);
-              pair_mixed2<false>(ii[r], b, 0, e2, p[r], q[r]);
+              pair_mixed2<kPhi, false>(ii[r], a, 0, e2, p[r], q[r]);
+              pair_mixed2<kPhi, false>(ii[r], b, 0, e2, p[r], q[r]);
             }
           }
         } else {
@@ -728,8 +735,8 @@ __device__ __forceinline__ void mixed_item(const ForceArgs& A, int n_act,
             load_j4(T, c, a, b);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-              pair_mixed2<true>(ii[r], a, c, e2, p[r], q[r], self[r]);
-              pair_mixed2<true>(ii[r], b, c + 2, e2, p[r], q[r], self[r]);
+              pair_mixed2<kPhi, true>(ii[r], a, c, e2, p[r], q[r], self[r]);
+              pair_mixed2<kPhi, true>(ii[r], b, c + 2, e2, p[r], q[r], self[r]);
             }
           }
         }
@@ -737,7 +744,7 @@ __device__ __forceinline__ void mixed_item(const ForceArgs& A, int n_act,
 #pragma unroll
       for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < (kPhi ? 4 : 3); ++c) {
           float a0, a1;
           upk(p[r][c], a0, a1);
           ds_add(s[r][c], a0 + a1);
@@ -750,7 +757,7 @@ __device__ __forceinline__ void mixed_item(const ForceArgs& A, int n_act,
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+      for (int c = 0; c < (kPhi ? 4 : 3); ++c)
         ds_add(s[r][c], DS{__shfl_xor_sync(kFull, s[r][c].hi, o),
                            __shfl_xor_sync(kFull, s[r][c].lo, o)});
       q[r] = fmaxf(q[r], __shfl_xor_sync(kFull, q[r], o));
@@ -767,17 +774,17 @@ __device__ __forceinline__ void mixed_item(const ForceArgs& A, int n_act,
     for (int c = 0; c < 4; ++c)
       x[c] = DS{second ? s[1][c].hi : s[0][c].hi,
                 second ? s[1][c].lo : s[0][c].lo};
-    write_partial(A, n_act, split, g * IG + (second ? IG / 2 : 0) + il,
+    write_partial<kPhi>(A, n_act, split, g * IG + (second ? IG / 2 : 0) + il,
                   to_double(x[0]), to_double(x[1]), to_double(x[2]),
                   -to_double(x[3]), to_double(second ? q[1] : q[0]));
   }
 }
 
-template <int JG>
+template <int JG, bool kPhi>
 __device__ void mixed_items(const ForceArgs& A, int n_act, const Plan& P,
                             MixTile<kTileMix>& T) {
   for (int w = blockIdx.x; w < P.n_g * P.S; w += gridDim.x)
-    mixed_item<JG>(A, n_act, P, w / P.S, w % P.S, T);
+    mixed_item<JG, kPhi>(A, n_act, P, w / P.S, w % P.S, T);
 }
 
 // Reduce the JG j-lane partial sums of each body in a fixed-order tree in

@@ -173,7 +173,7 @@ __global__ void ens_predict_kernel(Bodies B, Params P, Ens E, History prev) {
       const long long nt = tj + dtj;
       act = (nt == tn);
       if (nt < tn) atomicOr(&ctl->err, kErrInvariant);
-      predict_body(B, P, prev, j, tj, tn, pass, act, L);
+      predict_body(B, P, prev, j, j, tj, tn, pass, act, L);
     }
   }
   // lanes of one cluster share one atomic on the cluster's counter
@@ -534,8 +534,8 @@ __device__ void ens_tiled_item(const ForceArgs& A, int n_act, const Plan& P,
           for (int u = 0; u < U; ++u) {
             J2 a, b;
             load_j4(T, c0 + 4 * JG * u, a, b);
-            pair_mixed2<false>(ii, a, 0, e2, p, q);
-            pair_mixed2<false>(ii, b, 0, e2, p, q);
+            pair_mixed2<true, false>(ii, a, 0, e2, p, q);
+            pair_mixed2<true, false>(ii, b, 0, e2, p, q);
           }
         } else {
 #pragma unroll 1
@@ -543,8 +543,9 @@ __device__ void ens_tiled_item(const ForceArgs& A, int n_act, const Plan& P,
             const int c = c0 + 4 * JG * u;
             J2 a, b;
             load_j4(T, c, a, b);
-            pair_mixed2<true>(ii, a, c, e2, p, q, self);
-            pair_mixed2<true>(ii, b, c + 2, e2, p, q, self);
+            pair_mixed2<true, true>(ii, a, c, e2, p, q, self);
+            pair_mixed2<true, true>(ii, b, c + 2, e2, p, q,
+                                    self);
           }
         }
       }

@@ -27,7 +27,7 @@
 #include <mutex>
 #include <vector>
 
-#include "force_device.cuh"
+#include "force_far.cuh"
 #include "step_device.cuh"
 
 namespace tsbts {
@@ -144,16 +144,43 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// kPhi: the potential is summed (26 against 25 FMA-pipe operations; the
+// integrator does not read it). kSorted: bodies in spatial order, large
+// active sets by far_item.
+template <bool kPhi, bool kSorted>
 __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
     force_mixed_kernel(const __grid_constant__ ForceArgs A,
                        const __grid_constant__ PlanTable PT) {
+  union Sm {
+    FarSm far;
+    MixTile<kTileMix> tile;
+    float red[9][kThreads];
+  };
+  __shared__ __align__(16) unsigned char
+      smem[kSorted ? sizeof(Sm)
+                   : (sizeof(MixTile<kTileMix>) > sizeof(float[9][kThreads])
+                          ? sizeof(MixTile<kTileMix>)
+                          : sizeof(float[9][kThreads]))];
   int n_act = 0;
   if (!force_prologue(A, n_act)) return;
+  if constexpr (kSorted) {
+    if (n_act >= A.far_min && normal_eps2(A.eps2f)) {
+      FarSm& far = *reinterpret_cast<FarSm*>(smem);
+      const int S = far_splits(n_act, A.n, gridDim.x, A.part_cap);
+      if (blockIdx.x == 0 && threadIdx.x == 0 && A.nsplit_out)
+        *A.nsplit_out = S;
+      const int items = (n_act + 255) / 256 * S;
+      if (A.amask && blockIdx.x < items) rank_setup(A, far);
+      for (int w = blockIdx.x; w < items; w += gridDim.x)
+        far_item<kPhi>(A, n_act, w / S, w % S, S, far);
+      return;
+    }
+  }
   const Plan P = launch_plan(A, PT, n_act, 1);
   if (blockIdx.x == 0 && threadIdx.x == 0 && A.nsplit_out)
     *A.nsplit_out = P.S;
-  __shared__ MixTile<kTileMix> T;
-  __shared__ float red[9][kThreads];
+  // (a launch runs one form: staged tiles and the lanes' sums share memory)
+  float(*red)[kThreads] = reinterpret_cast<float(*)[kThreads]>(smem);
   if (P.direct && P.ig <= 32) {
     // direct loads serve the narrow groups
     switch (P.ig) {
@@ -166,13 +193,14 @@ __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
     }
     return;
   }
+  MixTile<kTileMix>& T = *reinterpret_cast<MixTile<kTileMix>*>(smem);
   switch (P.ig) {
-    case 256: mixed_items<1>(A, n_act, P, T); break;
-    case 128: mixed_items<2>(A, n_act, P, T); break;
-    case 64: mixed_items<4>(A, n_act, P, T); break;
-    case 32: mixed_items<8>(A, n_act, P, T); break;
-    case 16: mixed_items<16>(A, n_act, P, T); break;
-    default: mixed_items<32>(A, n_act, P, T); break;
+    case 256: mixed_items<1, kPhi>(A, n_act, P, T); break;
+    case 128: mixed_items<2, kPhi>(A, n_act, P, T); break;
+    case 64: mixed_items<4, kPhi>(A, n_act, P, T); break;
+    case 32: mixed_items<8, kPhi>(A, n_act, P, T); break;
+    case 16: mixed_items<16, kPhi>(A, n_act, P, T); break;
+    default: mixed_items<32, kPhi>(A, n_act, P, T); break;
   }
 }
 
@@ -189,8 +217,8 @@ constexpr int kFewFinalize = 2048;
 constexpr int kFinalizeThreads = 64;
 
 __global__ void __launch_bounds__(kFinalizeThreads)
-    force_finalize_kernel(const double* part, int S, int n_act, double* a,
-                          double* phi, double* q) {
+    force_finalize_kernel(const double* part, int S, int n_act,
+                          const int* pos, double* a, double* phi, double* q) {
   const int k = blockIdx.x * kFinalizeThreads + threadIdx.x;
   if (k >= n_act) return;
   double s[4];
@@ -203,11 +231,12 @@ __global__ void __launch_bounds__(kFinalizeThreads)
       s[c] = __dadd_rn(s[c], p[(long long)c * n_act + k]);
     qq = fmax(qq, p[4LL * n_act + k]);
   }
-  a[3 * (long long)k + 0] = s[0];
-  a[3 * (long long)k + 1] = s[1];
-  a[3 * (long long)k + 2] = s[2];
-  phi[k] = s[3];
-  q[k] = qq;
+  const int o = pos ? pos[k] : k;
+  a[3 * (long long)o + 0] = s[0];
+  a[3 * (long long)o + 1] = s[1];
+  a[3 * (long long)o + 2] = s[2];
+  phi[o] = s[3];
+  q[o] = qq;
 }
 
 __global__ void __launch_bounds__(kFinalizeThreads)
@@ -271,8 +300,8 @@ ForceLaunch force_launch_shape(int precision, int device) {
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (precision)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, force_mixed_kernel,
-                                                  kThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per_sm, force_mixed_kernel<true, false>, kThreads, 0);
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, force_fp64_kernel,
                                                   kThreads, 0);
@@ -309,8 +338,13 @@ cudaError_t launch_force(int precision, const ForceArgs& fa,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  if (precision)
-    return cudaLaunchKernelEx(&cfg, force_mixed_kernel, fa, pt ? *pt : none);
+  if (precision) {
+    auto* k = fa.no_phi ? (fa.meta ? force_mixed_kernel<false, true>
+                                   : force_mixed_kernel<false, false>)
+                        : (fa.meta ? force_mixed_kernel<true, true>
+                                   : force_mixed_kernel<true, false>);
+    return cudaLaunchKernelEx(&cfg, k, fa, pt ? *pt : none);
+  }
   if (fa.exact) {
     cfg.gridDim = dim3(fl.sms);
     return cudaLaunchKernelEx(&cfg, force_exact_kernel, fa);
@@ -488,16 +522,51 @@ cudaError_t autotune_mixed_plans(int device, const ForceArgs& base,
 }
 
 cudaError_t launch_force_finalize(const double* part, int S, int n_act,
-                                  double* a, double* phi, double* q,
-                                  cudaStream_t s) {
+                                  const int* pos, double* a, double* phi,
+                                  double* q, cudaStream_t s) {
   if (n_act <= 0) return cudaSuccess;
   constexpr int T = kFinalizeThreads;
-  if (S > 2 && n_act <= kFewFinalize)
+  if (S > 2 && n_act <= kFewFinalize && !pos)
     force_finalize_warp_kernel<<<(32 * n_act + T - 1) / T, T, 0, s>>>(
         part, S, n_act, a, phi, q);
   else
     force_finalize_kernel<<<(unsigned)((n_act + T - 1LL) / T), T, 0, s>>>(
-        part, S, n_act, a, phi, q);
+        part, S, n_act, pos, a, phi, q);
+  return cudaGetLastError();
+}
+
+int far_splits_host(int n_act, int n, int grid, long long part_cap) {
+  return far_splits(n_act, n, grid, part_cap);
+}
+
+__global__ void __launch_bounds__(256)
+    pack_sorted_kernel(int n, const int* order, const double* m,
+                       const double* r, const double* v, float4* jhi,
+                       float4* jlo, float4* jv, float4* meta) {
+  const int p = blockIdx.x * 256 + threadIdx.x;
+  float4 h = {}, u = {};
+  if (p < n) {
+    const long long j = order[p];
+    const double x = r[3 * j], y = r[3 * j + 1], z = r[3 * j + 2];
+    const float xh = (float)x, yh = (float)y, zh = (float)z;
+    h = make_float4(xh, yh, zh, (float)m[j]);
+    u = make_float4((float)v[3 * j], (float)v[3 * j + 1],
+                    (float)v[3 * j + 2], 0.f);
+    jhi[p] = h;
+    jlo[p] = make_float4((float)(x - (double)xh), (float)(y - (double)yh),
+                         (float)(z - (double)zh), 0.f);
+    jv[p] = u;
+  }
+  if ((p & ~31) < n)
+    store_subtile(meta, p / 32, p < n, h.x, h.y, h.z, u.x, u.y, u.z, h.w);
+}
+
+cudaError_t launch_pack_sorted(int n, const int* order, const double* m,
+                               const double* r, const double* v, float4* jhi,
+                               float4* jlo, float4* jv, float4* meta,
+                               cudaStream_t s) {
+  pack_sorted_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, order, m, r, v, jhi,
+                                                     jlo, jv, meta);
   return cudaGetLastError();
 }
 

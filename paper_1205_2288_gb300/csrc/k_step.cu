@@ -16,6 +16,7 @@
 // next multiple of the smallest populated step after the current block
 // time, and a per-level body count (updated by the correction)
 // replaces the paper's sort by block time.
+#include "force_far.cuh"
 #include "step_device.cuh"
 #include "tsbts_kernels.cuh"
 
@@ -75,6 +76,7 @@ __global__ void pass_setup_kernel(Bodies B, Params P, History cur) {
 // steps 3-4; Eq. 2; time-symmetric interpolation in passes >= 1).
 // ---------------------------------------------------------------------
 
+template <bool kSorted>
 __global__ void select_predict_kernel(Bodies B, Params P, History HA,
                                       History HB, int p) {
   __shared__ long long s_tn;
@@ -86,7 +88,8 @@ __global__ void select_predict_kernel(Bodies B, Params P, History HA,
   // this body's inputs, loaded before the block time and the pass are
   // known (the segment cache too: it is not used in the first pass), so
   // that every load of the kernel is in flight at once
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = kSorted && slot < B.n ? B.order[slot] : slot;
   long long tj = 0, dtj = 0;
   PredIn L;
   if (j < B.n) {
@@ -134,15 +137,30 @@ __global__ void select_predict_kernel(Bodies B, Params P, History HA,
     const long long nt = tj + dtj;
     act = (nt == tn);
     if (nt < tn) atomicOr(&ctl->err, kErrInvariant);
-    predict_body(B, P, prev, j, tj, tn, pass, act, L);
+    predict_body(B, P, prev, j, slot, tj, tn, pass, act, L);
   }
-  // compaction of the active list (order within a step is arbitrary)
+  // compaction of the active list (order within a step is arbitrary; in
+  // spatial order a force launch on many bodies lists them by the masks)
   const unsigned bal = __ballot_sync(kFull, act);
   const int lane = threadIdx.x & 31;
+  if (kSorted && slot - lane < B.n) {
+    if (lane == 0) B.amask[slot / 32] = bal;
+    float4 h = {}, v = {};
+    if (slot < B.n) {
+      h = B.jhi[slot];
+      v = B.jv[slot];
+    }
+    store_subtile(B.meta, slot / 32, slot < B.n, h.x, h.y, h.z, v.x, v.y, v.z,
+                  h.w);
+  }
   int base = 0;
   if (lane == 0 && bal) base = atomicAdd(&ctl->slot[p].cnt, __popc(bal));
   base = __shfl_sync(kFull, base, 0);
-  if (act) B.act[base + __popc(bal & ((1u << lane) - 1u))] = j;
+  if (act) {
+    const int k = base + __popc(bal & ((1u << lane) - 1u));
+    B.act[k] = j;
+    if (kSorted) B.aslot[k] = slot;
+  }
 }
 
 // ---------------------------------------------------------------------
@@ -512,7 +530,7 @@ __global__ void init_jdata_kernel(Bodies B, Params P) {
       rp[c] = B.r[c][j];
       vp[c] = B.v[c][j];
     }
-    store_prediction(B, P, j, rp, vp);
+    store_prediction(B, P, j, j, rp, vp);
   }
 }
 
@@ -661,7 +679,11 @@ cudaError_t launch_select_predict(const Bodies& B, const Params& P,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, select_predict_kernel, B, P, HA, HB, p);
+  if (B.order)
+    return cudaLaunchKernelEx(&cfg, select_predict_kernel<true>, B, P, HA, HB,
+                              p);
+  return cudaLaunchKernelEx(&cfg, select_predict_kernel<false>, B, P, HA, HB,
+                            p);
 }
 
 cudaError_t launch_correct(const Bodies& B, const Params& P,

@@ -50,9 +50,10 @@ __device__ __forceinline__ float to_float(double x) {
 }
 
 // j data of the force kernels at the block time: FP64 arrays or the packed
-// double-single records of the mixed path
+// double-single records of the mixed path (body j's at index slot)
 __device__ __forceinline__ void store_prediction(const Bodies& B,
                                                  const Params& P, int j,
+                                                 int slot,
                                                  const double rp[3],
                                                  const double vp[3]) {
   if (P.precision == 0) {
@@ -63,9 +64,9 @@ __device__ __forceinline__ void store_prediction(const Bodies& B,
   } else {
     float h[3], l[3];
     for (int c = 0; c < 3; ++c) split_ds(rp[c], h[c], l[c]);
-    B.jhi[j] = make_float4(h[0], h[1], h[2], B.mf[j]);
-    B.jlo[j] = make_float4(l[0], l[1], l[2], 0.f);
-    B.jv[j] = make_float4(to_float(vp[0]), to_float(vp[1]), to_float(vp[2]),
+    B.jhi[slot] = make_float4(h[0], h[1], h[2], B.mf[j]);
+    B.jlo[slot] = make_float4(l[0], l[1], l[2], 0.f);
+    B.jv[slot] = make_float4(to_float(vp[0]), to_float(vp[1]), to_float(vp[2]),
                           0.f);
   }
 }
@@ -119,7 +120,8 @@ __device__ __forceinline__ void load_pred_in(const Bodies& B, int j,
 // tn leaves the segment. L holds the body's preloaded inputs.
 __device__ __forceinline__ void predict_body(const Bodies& B, const Params& P,
                                              const History& prev, int j,
-                                             long long tj, long long tn,
+                                             int slot, long long tj,
+                                             long long tn,
                                              int pass, bool act, PredIn& L) {
   double rp[3], vp[3];
   bool have = false;
@@ -199,7 +201,7 @@ __device__ __forceinline__ void predict_body(const Bodies& B, const Params& P,
       }
     }
   }
-  store_prediction(B, P, j, rp, vp);
+  store_prediction(B, P, j, slot, rp, vp);
 }
 
 // S split partial sums of active position k (layout [split][5][n_act]),

@@ -91,6 +91,13 @@ struct Bodies {
   float4* jlo;
   float4* jv;
   int* act;          // active list of the step
+  // spatially sorted runs (nullptr otherwise): body of each slot (the j
+  // records are stored by slot), bit masks of the step's active slots, the
+  // slots of act, and two float4 per 32 slots (force_far.cuh)
+  int* order;
+  unsigned* amask;
+  int* aslot;
+  float4* meta;
   int* cursor;       // per body: its last previous-pass record (CSR index)
                      // with tau <= the current block time
   int* hcnt;         // per body: records appended in the running pass
@@ -199,7 +206,28 @@ struct ForceArgs {
   double eps2;
   float eps2f;
   int exact;           // FP64: no j-split
+  // mixed: the potential's partial sums are not read (no_phi); bodies in
+  // spatial order (idx holds their slots) with the subtiles' summaries
+  // (force_far.cuh), used from far_min active bodies on (meta nullable).
+  // There the active slots in order are idx (amask nullptr), or those of
+  // the bit masks, and then their bodies order[slot] are written to act
+  int no_phi;
+  const float4* meta;
+  int far_min;
+  const unsigned* amask;
+  const int* order;
+  int* act;
 };
+
+// Bodies from which the mixed force keeps spatial order (integrator: sorted
+// once per era) or sorts (stand-alone call), and the fewest active ones, per
+// body, that take the far form. Below, reading the bodies through the order
+// in every prediction costs what the far pairs of large steps save: eras
+// against the unsorted force, 16384 bodies 109 and 98 ms, 25000 34.3 and
+// 31.5, 50000 84 and 98, 131072 263 and 389.
+constexpr int kSortMinBodies = 32768;
+constexpr int kSortMaxBodies = 1 << 20;
+constexpr int kFarMinShare = 16;
 
 // Measured work plans of the integrator's force launch, one per power-of-two
 // bucket of active counts (bucket b holds counts in (2^(b-1), 2^b], the last
@@ -397,10 +425,30 @@ cudaError_t autotune_mixed_plans(int device, const ForceArgs& base,
 cudaError_t launch_force(int precision, const ForceArgs& fa,
                          const ForceLaunch& fl, cudaStream_t s,
                          const PlanTable* pt = nullptr, bool pdl = false);
-// sum S split partials per active body into AoS a, phi, q
+// sum S split partials per active body into AoS a, phi, q (pos, nullable:
+// the row of each)
 cudaError_t launch_force_finalize(const double* part, int S, int n_act,
-                                  double* a, double* phi, double* q,
-                                  cudaStream_t s);
+                                  const int* pos, double* a, double* phi,
+                                  double* q, cudaStream_t s);
+// spatial order (k_sort.cu): keys a sort of n needs; order (and its inverse
+// slot, nullable) of bodies with coordinates x[i * stride] ...; part: 128
+// doubles; returns the number of launches
+int sort_capacity(long long n);
+int launch_spatial_order(int n, const double* x, const double* y,
+                         const double* z, int stride, double* part,
+                         unsigned long long* key, int* order, int* slot,
+                         cudaStream_t s);
+// idx[0..n_act) as ascending slots `list` with their positions `pos` in idx
+void launch_sorted_list(int n_act, const int* idx, const int* slot,
+                        unsigned long long* key, int* list, int* pos,
+                        cudaStream_t s);
+// split count of a far-form launch (force_far.cuh)
+int far_splits_host(int n_act, int n, int grid, long long part_cap);
+// mixed j records of AoS bodies by slot, with the subtiles' summaries
+cudaError_t launch_pack_sorted(int n, const int* order, const double* m,
+                               const double* r, const double* v, float4* jhi,
+                               float4* jlo, float4* jv, float4* meta,
+                               cudaStream_t s);
 // AoS (n, 3) -> packed j records for either precision
 cudaError_t launch_pack_aos(int precision, int n, const double* m,
                             const double* r, const double* v, double* sx,
