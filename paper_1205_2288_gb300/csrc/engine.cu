@@ -756,7 +756,8 @@ struct Scratch {
   unsigned long long* key = nullptr;
   float4* meta = nullptr;
   double* scale = nullptr;
-  int sort_cap = 0;       // bodies (and active bodies) it has room for
+  int sort_cap = 0;       // most bodies (and active bodies) of a sorted call
+  size_t sort_stride = 0; // ints of each of the four arrays
 };
 
 void free_sort(Scratch& S) {
@@ -769,6 +770,7 @@ void free_sort(Scratch& S) {
   S.meta = nullptr;
   S.scale = nullptr;
   S.sort_cap = 0;
+  S.sort_stride = 0;
 }
 
 // Whether a mixed force call sorts its bodies: the sorts of the bodies and of
@@ -1258,33 +1260,35 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
       ck(cudaMemcpy(S.iota, iota.data(), sizeof(int) * (size_t)ncap,
                     cudaMemcpyHostToDevice),
          "scratch");
+      if (ncap >= kSortMinBodies) {
+        // with the rest, so that no later call of this size allocates
+        const size_t cap = (size_t)std::min<int64_t>(
+            std::max<int64_t>(ncap, n_act), kSortMaxBodies);
+        ck(cudaMalloc(&S.sort_i, sizeof(int) * 4 * cap), "scratch");
+        ck(cudaMalloc(&S.key, sizeof(unsigned long long) *
+                                  (size_t)sort_capacity((long long)cap)),
+           "scratch");
+        ck(cudaMalloc(&S.meta, sizeof(float4) * 2 * (cap / 32 + 1)),
+           "scratch");
+        ck(cudaMalloc(&S.scale, sizeof(double) * 128), "scratch");
+        S.sort_cap = (int)cap;
+        S.sort_stride = cap;
+      }
       S.n_cap = ncap;
       S.part_cap = need_part;
     }
     const int ni = (int)n;
     double* x = S.soa;
     float4* j4 = S.j4;
-    const bool sorts = force_sorts(precision, n, n_act, eps);
+    const bool sorts = force_sorts(precision, n, n_act, eps) &&
+                       std::max(n, n_act) <= S.sort_cap;
     if (sorts) {
-      const int need = (int)std::max(n, n_act);
-      if (S.sort_cap < need) {
-        ck(cudaDeviceSynchronize(), "synchronize before scratch growth");
-        free_sort(S);
-        ck(cudaMalloc(&S.sort_i, sizeof(int) * 4 * (size_t)need), "scratch");
-        ck(cudaMalloc(&S.key, sizeof(unsigned long long) *
-                                  (size_t)sort_capacity(need)),
-           "scratch");
-        ck(cudaMalloc(&S.meta, sizeof(float4) * 2 * ((size_t)need / 32 + 1)),
-           "scratch");
-        ck(cudaMalloc(&S.scale, sizeof(double) * 128), "scratch");
-        S.sort_cap = need;
-      }
       int* order = S.sort_i;
-      int* slot = order + S.sort_cap;
+      int* slot = order + S.sort_stride;
       launch_spatial_order(ni, r, r + 1, r + 2, 3, S.scale, S.key, order,
                            slot, s);
-      launch_sorted_list((int)n_act, idx, slot, S.key, slot + S.sort_cap,
-                         slot + 2LL * S.sort_cap, s);
+      launch_sorted_list((int)n_act, idx, slot, S.key, slot + S.sort_stride,
+                         slot + 2 * S.sort_stride, s);
       ck(launch_pack_sorted(ni, order, m, r, v, j4, j4 + ni, j4 + 2LL * ni,
                             S.meta, s),
          "pack");
@@ -1315,12 +1319,7 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
                (exact_order == 1 || (exact_order < 0 && n <= 8192));
     fa.plan = plan_force(precision, fa.exact, (int)n_act, ni, fl,
                          S.part_cap);
-    if (sorts) {
-      fa.idx = S.sort_i + 2LL * S.sort_cap;
-      fa.meta = S.meta;
-      fa.far_min = 0;
-      fa.plan.S = far_splits_host((int)n_act, ni, fl.grid, S.part_cap);
-    } else if (precision == TSBTS_MIXED && ni <= (1 << 20)) {
+    if (precision == TSBTS_MIXED && ni <= (1 << 20)) {
       // measured plans: the first call for a new n tunes them on these j
       // records and caches the table for the process
       const std::vector<Plan>* tp = tuned_plans(dev, ni, fl.grid);
@@ -1334,8 +1333,16 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
            "force plan autotuning");
         tp = tuned_plans(dev, ni, fl.grid);
       }
-      if (tp && (long long)(*tp)[n_act].S * 5 * n_act <= S.part_cap)
+      // (repeated bodies may make the list longer than the table)
+      if (tp && n_act <= n &&
+          (long long)(*tp)[n_act].S * 5 * n_act <= S.part_cap)
         fa.plan = (*tp)[n_act];
+    }
+    if (sorts) {
+      fa.idx = S.sort_i + 2 * S.sort_stride;
+      fa.meta = S.meta;
+      fa.far_min = 0;
+      fa.plan.S = far_splits_host((int)n_act, ni, fl.grid, S.part_cap);
     }
     fa.has_plan = 1;
     if (std::getenv("TSBTS_PRINT_PLANS"))
@@ -1345,7 +1352,7 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
                    fa.plan.direct ? "direct" : "tiled");
     ck(launch_force(precision, fa, fl, s), "force");
     ck(launch_force_finalize(S.part, fa.exact ? 1 : fa.plan.S, (int)n_act,
-                             sorts ? S.sort_i + 3LL * S.sort_cap : nullptr,
+                             sorts ? S.sort_i + 3 * S.sort_stride : nullptr,
                              a, phi, q, s),
        "force finalize");
     return TSBTS_OK;

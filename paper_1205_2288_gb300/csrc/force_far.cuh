@@ -291,9 +291,11 @@ __device__ __forceinline__ void far_item(const ForceArgs& A, int n_act, int g,
       const float gz = box_gap(wb.lo[2], wb.hi[2], lo.z, hi.z);
       const float d2 = 0.9999f * fmaf(gx, gx, fmaf(gy, gy, gz * gz));
       is_far = d2 > rho2;
-      const float r2 = 1.f / (d2 + eps2), w = vmax + lo.w;
-      const float most = 1.0001f * fmaxf(w * w * r2, hi.w * r2 * sqrtf(r2));
-      no_crit = qm != ~0u && most <= __uint_as_float(qm);
+      // (both comparisons fail where a speed or mass is no number)
+      const float r2 = 1.0001f / (d2 + eps2), w = vmax + lo.w;
+      const float least = __uint_as_float(qm);
+      no_crit = qm != ~0u && w * w * r2 <= least &&
+                hi.w * r2 * sqrtf(r2) <= least;
     }
     const unsigned plain = __ballot_sync(kFull, no_crit);
     const unsigned fars = __ballot_sync(kFull, is_far) & plain;
