@@ -34,12 +34,13 @@ namespace tsbts {
 
 // Host choice of the work plan for n_act active bodies: tiled_plan in the
 // mixed path; in FP64, over i-group widths 128 .. 1 and split counts,
-// minimise the time of the busiest SM plus the consumer's cost of reading S
-// partial sums. The FP64 pipe is saturated by one block per SM, so an SM's
-// time is its number of items, whatever the number of resident blocks: 640
-// items on 152 SMs cost five items' time, not 4.2 (5000 of 20000 bodies: 5.85
-// ms with S chosen for the waves of the resident grid, 4.93 ms by items per
-// SM).
+// minimise the waves of the grid (two blocks per SM) times an item's time,
+// plus the consumer's cost of reading S partial sums. Few blocks per SM, each
+// with work: the FP64 pipe is saturated by one block, and of a grid of eight
+// per SM the blocks with work may share SMs while others idle (1024 of 131072
+// bodies ran at 11 G interactions/s, all of them at 22). 5000 of 20000
+// bodies: 5.85 ms with S chosen for the waves of eight blocks per SM, 4.61 ms
+// now.
 Plan plan_force(int precision, int exact, int n_act, int n,
                 const ForceLaunch& fl, long long part_cap) {
   Plan best = {kThreads, (n_act + kThreads - 1) / kThreads, 1, n, 0};
@@ -56,9 +57,9 @@ Plan plan_force(int precision, int exact, int n_act, int n,
     for (int S = 1; S <= smax; ++S) {
       if (S > 1 && (long long)S * 5 * n_act > part_cap) break;
       const long long chunk = (n + S - 1) / S;
-      const long long per_sm = (n_g * S + fl.sms - 1) / fl.sms;
+      const long long waves = (n_g * S + fl.grid - 1) / fl.grid;
       const double per_item = (double)((chunk + jg - 1) / jg) + 2.0;
-      const double cost = per_sm * per_item + 0.3 * S;
+      const double cost = 2 * waves * per_item + 0.3 * S;
       if (cost < best_cost) {
         best_cost = cost;
         best = Plan{ig, (int)n_g, S, (int)chunk, 0};
@@ -308,12 +309,12 @@ ForceLaunch force_launch_shape(int precision, int device) {
   if (sms < 1) sms = 1;
   if (per_sm < 1) per_sm = 1;
   ForceLaunch fl;
-  fl.grid = sms * per_sm;
+  fl.grid = precision ? sms * per_sm : 2 * sms;  // (plan_force)
   fl.sms = sms;
 
   fl.threads = kThreads;
   fl.tile_i = kThreads;
-  fl.part_cap = 5LL * fl.grid * kThreads;
+  fl.part_cap = 5LL * sms * per_sm * kThreads;
   if (cached) c[device] = fl;
   return fl;
 }
