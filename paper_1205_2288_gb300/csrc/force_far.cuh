@@ -20,9 +20,9 @@
 // A far pair then takes 13 FMA-pipe operations and about 31 register reads
 // instead of 26 and 57, a near one without the criterion 19 and 41. Of the
 // pairs of all of 131072 bodies three quarters are far, of 16384 a quarter.
-// All of 131072 bodies: 11.2 ms with both sorts, 14.65 in the unsorted form;
-// the start of their era 263 ms, 389 before. Errors against 64 bits are the
-// same (a 4e-8, phi 3e-8, q 1.1e-7).
+// All of 131072 bodies: 11.3 ms with both sorts, 14.65 in the unsorted form;
+// the start of their era 269 ms, 389 before. Errors against 64 bits (relative
+// 2-norms): a 2.7e-8 (3.2e-8 unsorted), phi 7e-9 (9e-9), q 1.1e-7 (1.1e-7).
 #pragma once
 
 #include "force_device.cuh"
@@ -306,57 +306,57 @@ __device__ __forceinline__ void far_item(const ForceArgs& A, int n_act, int g,
       const int e = sub >= 0 && sub % S == split ? sub / S - m0 : -1;
       selfs |= __reduce_or_sync(kFull, e >= 0 && e < ns ? 1u << e : 0u);
     }
-    for (int e0 = 0; e0 < ns; e0 += kStrip / kSubJ) {
+    // FP32 sums over one subtile, then folded: its bodies pull the same way,
+    // so that longer sums (256 j as in the unsorted form) would grow with
+    // each term and round 1.25 to 1.5 times as far from 64 bits
+    for (int e = 0; e < ns; ++e) {
       const f2 z = pk(0.f, 0.f);
       f2 p[2][4] = {{z, z, z, z}, {z, z, z, z}};
-      const int e1 = min(ns, e0 + kStrip / kSubJ);
-      for (int e = e0; e < e1; ++e) {
-        const int c0 = e * kSubJ;
-        if (fars >> e & 1) {
+      const int c0 = e * kSubJ;
+      if (fars >> e & 1) {
 #pragma unroll 2
-          for (int c = c0; c < c0 + kSubJ; c += 4) {
-            const ulonglong2 x = lds4(&T.cx[c]), y = lds4(&T.cy[c]),
-                             zz = lds4(&T.cz[c]), m = lds4(&T.t.m[c]);
+        for (int c = c0; c < c0 + kSubJ; c += 4) {
+          const ulonglong2 x = lds4(&T.cx[c]), y = lds4(&T.cy[c]),
+                           zz = lds4(&T.cz[c]), m = lds4(&T.t.m[c]);
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              pair_far2<kPhi>(ci[r], x.x, y.x, zz.x, m.x, e2, p[r]);
-              pair_far2<kPhi>(ci[r], x.y, y.y, zz.y, m.y, e2, p[r]);
-            }
+          for (int r = 0; r < 2; ++r) {
+            pair_far2<kPhi>(ci[r], x.x, y.x, zz.x, m.x, e2, p[r]);
+            pair_far2<kPhi>(ci[r], x.y, y.y, zz.y, m.y, e2, p[r]);
           }
-        } else if ((plain & ~selfs) >> e & 1) {
+        }
+      } else if ((plain & ~selfs) >> e & 1) {
 #pragma unroll 2
-          for (int c = c0; c < c0 + kSubJ; c += 4) {
-            J2 a, b;
-            load_j4(T.t, c, a, b);
+        for (int c = c0; c < c0 + kSubJ; c += 4) {
+          J2 a, b;
+          load_j4(T.t, c, a, b);
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              pair_mixed2<kPhi, false, false>(ii[r], a, 0, e2, p[r], q[r]);
-              pair_mixed2<kPhi, false, false>(ii[r], b, 0, e2, p[r], q[r]);
-            }
+          for (int r = 0; r < 2; ++r) {
+            pair_mixed2<kPhi, false, false>(ii[r], a, 0, e2, p[r], q[r]);
+            pair_mixed2<kPhi, false, false>(ii[r], b, 0, e2, p[r], q[r]);
           }
-        } else if (selfs >> e & 1) {
-          const int base = (split + S * (m0 + e)) * kSubJ - c0;
+        }
+      } else if (selfs >> e & 1) {
+        const int base = (split + S * (m0 + e)) * kSubJ - c0;
 #pragma unroll 1
-          for (int c = c0; c < c0 + kSubJ; c += 4) {
-            J2 a, b;
-            load_j4(T.t, c, a, b);
+        for (int c = c0; c < c0 + kSubJ; c += 4) {
+          J2 a, b;
+          load_j4(T.t, c, a, b);
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              const int self = own[r] - base;
-              pair_mixed2<kPhi, true>(ii[r], a, c, e2, p[r], q[r], self);
-              pair_mixed2<kPhi, true>(ii[r], b, c + 2, e2, p[r], q[r], self);
-            }
+          for (int r = 0; r < 2; ++r) {
+            const int self = own[r] - base;
+            pair_mixed2<kPhi, true>(ii[r], a, c, e2, p[r], q[r], self);
+            pair_mixed2<kPhi, true>(ii[r], b, c + 2, e2, p[r], q[r], self);
           }
-        } else {
+        }
+      } else {
 #pragma unroll 2
-          for (int c = c0; c < c0 + kSubJ; c += 4) {
-            J2 a, b;
-            load_j4(T.t, c, a, b);
+        for (int c = c0; c < c0 + kSubJ; c += 4) {
+          J2 a, b;
+          load_j4(T.t, c, a, b);
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              pair_mixed2<kPhi, false>(ii[r], a, 0, e2, p[r], q[r]);
-              pair_mixed2<kPhi, false>(ii[r], b, 0, e2, p[r], q[r]);
-            }
+          for (int r = 0; r < 2; ++r) {
+            pair_mixed2<kPhi, false>(ii[r], a, 0, e2, p[r], q[r]);
+            pair_mixed2<kPhi, false>(ii[r], b, 0, e2, p[r], q[r]);
           }
         }
       }

@@ -224,7 +224,7 @@ struct ForceArgs {
 // body, that take the far form. Below, reading the bodies through the order
 // in every prediction costs what the far pairs of large steps save: eras
 // against the unsorted force, 16384 bodies 109 and 98 ms, 25000 34.3 and
-// 31.5, 50000 84 and 98, 131072 263 and 389.
+// 31.5, 50000 84 and 98, 131072 269 and 389.
 constexpr int kSortMinBodies = 32768;
 constexpr int kSortMaxBodies = 1 << 20;
 constexpr int kFarMinShare = 16;
