@@ -237,7 +237,10 @@ void tsbts_destroy(tsbts_ctx* ctx);
  * asynchronous: outputs are ready when the stream reaches this point.
  * Scratch memory (packed j records and j-split partial sums) is allocated
  * by the library on first use per device, grown as needed and kept until
- * tsbts_release_scratch. TSBTS_ERR_ARG: n < 1, n_act < 0, n or n_act above
+ * tsbts_release_scratch. Calls on different streams share it: each waits on
+ * the GPU for the one before it, also among the calls of one stream
+ * capture. Launches of a captured graph are the caller's to order against
+ * other calls. TSBTS_ERR_ARG: n < 1, n_act < 0, n or n_act above
  * 2^31 - 1, or eps < 0. */
 int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
                 const double* r, const double* v, double eps, int64_t n_act,

@@ -758,6 +758,46 @@ struct Scratch {
   double* scale = nullptr;
   int sort_cap = 0;       // most bodies (and active bodies) of a sorted call
   size_t sort_stride = 0; // ints of each of the four arrays
+  // the end of the last call's work, outside and inside stream captures
+  // (of the capture cap_id)
+  cudaEvent_t last = nullptr, cap_last = nullptr;
+  unsigned long long cap_id = 0;
+};
+
+void free_events(Scratch& S) {
+  if (S.last) cudaEventDestroy(S.last);
+  if (S.cap_last) cudaEventDestroy(S.cap_last);
+  S.last = S.cap_last = nullptr;
+}
+
+// A call's turn on the scratch memory, held with g_scratch_mu: the stream
+// waits for the work of the call before, whatever stream that was on (two
+// calls at once would overwrite each other's j records, order and partial
+// sums, and follow each other's slots out of the arrays), and the end of this
+// call's work is marked for the next one, also where the call fails half
+// way. Inside a stream capture the calls of that capture are ordered the
+// same way; a captured graph's launches are the caller's to order.
+class ScratchTurn {
+ public:
+  ScratchTurn(Scratch& S, cudaStream_t s) : s_(s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    ck(cudaStreamGetCaptureInfo(s, &st, &id), "capture state");
+    const bool capturing = st == cudaStreamCaptureStatusActive;
+    e_ = capturing ? S.cap_last : S.last;
+    if (!capturing || id == S.cap_id)
+      ck(cudaStreamWaitEvent(s, e_, 0), "wait for the scratch memory");
+    if (capturing) S.cap_id = id;
+  }
+  ~ScratchTurn() {
+    if (cudaEventRecord(e_, s_) != cudaSuccess) cudaGetLastError();
+  }
+  ScratchTurn(const ScratchTurn&) = delete;
+  ScratchTurn& operator=(const ScratchTurn&) = delete;
+
+ private:
+  cudaStream_t s_;
+  cudaEvent_t e_;
 };
 
 void free_sort(Scratch& S) {
@@ -1248,7 +1288,14 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
       cudaFree(S.nsplit);
       cudaFree(S.iota);
       free_sort(S);
+      const Scratch old = S;
       S = Scratch{};
+      S.last = old.last;
+      S.cap_last = old.cap_last;
+      S.cap_id = old.cap_id;
+      for (cudaEvent_t* e : {&S.last, &S.cap_last})
+        if (!*e)
+          ck(cudaEventCreateWithFlags(e, cudaEventDisableTiming), "scratch");
       const int ncap = (int)std::max<int64_t>(n, S.n_cap);
       ck(cudaMalloc(&S.soa, sizeof(double) * 7 * (size_t)ncap), "scratch");
       ck(cudaMalloc(&S.j4, sizeof(float4) * 3 * (size_t)ncap), "scratch");
@@ -1277,6 +1324,7 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
       S.n_cap = ncap;
       S.part_cap = need_part;
     }
+    const ScratchTurn turn(S, s);
     const int ni = (int)n;
     double* x = S.soa;
     float4* j4 = S.j4;
@@ -1376,6 +1424,7 @@ int tsbts_release_scratch(void) {
   cudaFree(S.nsplit);
   cudaFree(S.iota);
   free_sort(S);
+  free_events(S);
   S = Scratch{};
   return TSBTS_OK;
 }
