@@ -644,10 +644,12 @@ int init_common(tsbts_ctx* c, int64_t n, const double* m, const double* r,
     c->correct_grid = std::max(1, std::min(c->sms * 32, (c->n + 31) / 32));
     c->ensemble = false;
     c->nc = 0;
-    // large mixed systems keep their j records in spatial order
+    // large mixed systems keep their j records in spatial order (the far
+    // form takes an eps^2 that is a normal float)
     setup_bodies(c, (int)n,
                  c->cfg.precision == TSBTS_MIXED && !ens &&
-                     n >= kSortMinBodies && n <= kSortMaxBodies);
+                     n >= kSortMinBodies && n <= kSortMaxBodies &&
+                     normal_eps2((float)(eps * eps)));
     if (ens) {
       c->pt = PlanTable{};
       setup_ensemble(c, *ens);
@@ -822,7 +824,7 @@ bool force_sorts(int precision, int64_t n, int64_t n_act, double eps) {
   return precision == TSBTS_MIXED && n >= kSortMinBodies &&
          n <= kSortMaxBodies && n_act >= n / kFarMinShare &&
          n_act <= kSortMaxBodies && n * n_act >= (1LL << 31) &&
-         eps2 >= 1.17549435e-38f;
+         normal_eps2(eps2);
 }
 std::mutex g_scratch_mu;
 std::vector<Scratch> g_scratch;

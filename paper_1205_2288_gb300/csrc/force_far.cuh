@@ -331,8 +331,8 @@ __device__ __forceinline__ void far_item(const ForceArgs& A, int n_act, int g,
           load_j4(T.t, c, a, b);
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
-            pair_mixed2<kPhi, false, false>(ii[r], a, 0, e2, p[r], q[r]);
-            pair_mixed2<kPhi, false, false>(ii[r], b, 0, e2, p[r], q[r]);
+            pair_mixed2<kPhi, false, false, false>(ii[r], a, 0, e2, p[r], q[r]);
+            pair_mixed2<kPhi, false, false, false>(ii[r], b, 0, e2, p[r], q[r]);
           }
         }
       } else if (selfs >> e & 1) {
@@ -344,8 +344,9 @@ __device__ __forceinline__ void far_item(const ForceArgs& A, int n_act, int g,
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
             const int self = own[r] - base;
-            pair_mixed2<kPhi, true>(ii[r], a, c, e2, p[r], q[r], self);
-            pair_mixed2<kPhi, true>(ii[r], b, c + 2, e2, p[r], q[r], self);
+            pair_mixed2<kPhi, true, true>(ii[r], a, c, e2, p[r], q[r], self);
+            pair_mixed2<kPhi, true, true>(ii[r], b, c + 2, e2, p[r], q[r],
+                                          self);
           }
         }
       } else {
@@ -355,8 +356,8 @@ __device__ __forceinline__ void far_item(const ForceArgs& A, int n_act, int g,
           load_j4(T.t, c, a, b);
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
-            pair_mixed2<kPhi, false>(ii[r], a, 0, e2, p[r], q[r]);
-            pair_mixed2<kPhi, false>(ii[r], b, 0, e2, p[r], q[r]);
+            pair_mixed2<kPhi, false, false>(ii[r], a, 0, e2, p[r], q[r]);
+            pair_mixed2<kPhi, false, false>(ii[r], b, 0, e2, p[r], q[r]);
           }
         }
       }

@@ -835,12 +835,12 @@ __device__ __forceinline__ void vjp_j_f64(const VjpArgs& A, int b, VjpSm& sm) {
 // pairs; every FMA-pipe operation works on two sources at once (f32x2).
 // A tile is padded to a multiple of 4 tpt with neutral sources (zero mass
 // or zero lam, far away), so every lane runs the same packed loop. The warp
-// ORs the loop iterations that hold one of its targets; those (and all of
-// them where eps^2 is no normal float) run the masked form, where a target's
-// own pair gets 1/s = 0 and adds exact zeros, and the square root takes
-// subnormals; both forms round alike. (With every tile that holds a target
-// masked as a whole, a step on all bodies ran a quarter of its loops
-// masked.)
+// ORs the loop iterations that hold one of its targets; those run the masked
+// form, where a target's own pair gets 1/s = 0 and adds exact zeros. kSafe:
+// eps^2 is no normal float, and the other iterations take the square root
+// that handles subnormals, as the masked ones do; all forms round alike.
+// (With every tile that holds a target masked as a whole, a step on all
+// bodies ran a quarter of its loops masked.)
 constexpr int kVjpTile = TSBTS_VJP_TILE;
 constexpr float kFar = 1.0e18f;
 
@@ -864,7 +864,7 @@ __device__ __forceinline__ ulonglong2 ld4(const float* p) {
 
 // two sources (tile slots c, c + 1) on one active body: ii holds the
 // target's hi (0..2), lo (3..5) and lam (6..8), each broadcast to a pair
-template <bool kMask>
+template <bool kSafe, bool kMask>
 __device__ __forceinline__ void pair_vjp_i2(const f2 (&ii)[9], f2 xh, f2 yh,
                                             f2 zh, f2 m, f2 xl, f2 yl, f2 zl,
                                             int c, int self, f2 e2, f2& W,
@@ -875,7 +875,7 @@ __device__ __forceinline__ void pair_vjp_i2(const f2 (&ii)[9], f2 xh, f2 yh,
   const f2 s2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
   float s0, s1;
   upk(s2, s0, s1);
-  float r0 = rsqrt_of<kMask>(s0), r1 = rsqrt_of<kMask>(s1);
+  float r0 = rsqrt_of<kSafe>(s0), r1 = rsqrt_of<kSafe>(s1);
   if (kMask) {
     if (c == self) r0 = 0.f;
     if (c + 1 == self) r1 = 0.f;
@@ -893,7 +893,7 @@ __device__ __forceinline__ void pair_vjp_i2(const f2 (&ii)[9], f2 xh, f2 yh,
 
 // two active sources (tile slots c, c + 1) on one body: jj holds the
 // target's hi (0..2) and lo (3..5)
-template <bool kMask>
+template <bool kSafe, bool kMask>
 __device__ __forceinline__ void pair_vjp_j2(const f2 (&jj)[6], f2 xh, f2 yh,
                                             f2 zh, f2 xl, f2 yl, f2 zl, f2 lx,
                                             f2 ly, f2 lz, int c, int self,
@@ -905,7 +905,7 @@ __device__ __forceinline__ void pair_vjp_j2(const f2 (&jj)[6], f2 xh, f2 yh,
   const f2 s2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
   float s0, s1;
   upk(s2, s0, s1);
-  float r0 = rsqrt_of<kMask>(s0), r1 = rsqrt_of<kMask>(s1);
+  float r0 = rsqrt_of<kSafe>(s0), r1 = rsqrt_of<kSafe>(s1);
   if (kMask) {
     if (c == self) r0 = 0.f;
     if (c + 1 == self) r1 = 0.f;
@@ -931,9 +931,7 @@ __device__ __forceinline__ float hsum(f2 x) {
 // the own source sc (tile slot, < 0: none) of a target of this warp; at
 // most kVjpTile / 4 = 128 iterations, whose numbers are taken modulo 64 (the
 // loop rotates the mask; a masked iteration that needs none is only slower)
-__device__ __forceinline__ unsigned long long self_mask(int sc, int step,
-                                                        bool normal) {
-  if (!normal) return ~0ULL;
+__device__ __forceinline__ unsigned long long self_mask(int sc, int step) {
   const int own = sc < 0 ? -1 : sc / step & 63;
   const unsigned lo =
       __reduce_or_sync(kFull, own >= 0 && own < 32 ? 1u << own : 0u);
@@ -942,6 +940,7 @@ __device__ __forceinline__ unsigned long long self_mask(int sc, int step,
   return ((unsigned long long)hi << 32) | lo;
 }
 
+template <bool kSafe>
 __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
                                             VjpSmem& T0, VjpSm& sm) {
   const VjpSide& V = A.V.si;
@@ -957,7 +956,6 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
                     pk(lm.x, lm.x), pk(lm.y, lm.y), pk(lm.z, lm.z)};
   const f2 e2 = pk(A.eps2f, A.eps2f);
   const int step = 4 * V.tpt;
-  const bool normal = normal_eps2(A.eps2f);
   DS dacc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};  // W, U
   VjpTileI& T = T0.i;
   for (int jt = B.beg; jt < B.end; jt += kVjpTile) {
@@ -978,7 +976,7 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
     const bool self_here = B.live && bi >= jt && bi < jt + cnt;
     const int sc = self_here ? bi - jt : -1;
     f2 W = pk(0.f, 0.f), Ux = W, Uy = W, Uz = W;
-    unsigned long long mask = self_mask(sc, step, normal);
+    unsigned long long mask = self_mask(sc, step);
     int c = 4 * B.lane;
     // (cntp is a whole number of steps; two to an unrolled iteration)
     for (int m = 0; m < iters; m += kVjpUnroll,
@@ -991,9 +989,9 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
                            zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
                            xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
                            zl = ld4(&T.zl[c]);
-          pair_vjp_i2<false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c,
+          pair_vjp_i2<kSafe, false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c,
                              -1, e2, W, Ux, Uy, Uz);
-          pair_vjp_i2<false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+          pair_vjp_i2<kSafe, false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
                              -1, e2, W, Ux, Uy, Uz);
         }
       } else {
@@ -1003,9 +1001,9 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
                            zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
                            xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
                            zl = ld4(&T.zl[c]);
-          pair_vjp_i2<true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
+          pair_vjp_i2<true, true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
                             e2, W, Ux, Uy, Uz);
-          pair_vjp_i2<true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+          pair_vjp_i2<true, true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
                             sc, e2, W, Ux, Uy, Uz);
         }
       }
@@ -1020,6 +1018,7 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
   vjp_finish<0>(A, V, B, A.n_act, acc, A.O.part_i, A.O.cnt_i, sm);
 }
 
+template <bool kSafe>
 __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
                                             VjpSmem& T0, VjpSm& sm) {
   const VjpSide& V = A.V.sj;
@@ -1034,7 +1033,6 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
   const f2 e2 = pk(A.eps2f, A.eps2f);
   const f2 m3 = pk(-3.f, -3.f);
   const int step = 4 * V.tpt;
-  const bool normal = normal_eps2(A.eps2f);
   DS dacc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};  // G, Z
   VjpTileJ& T = T0.j;
   for (int kt = B.beg; kt < B.end; kt += kVjpTile) {
@@ -1058,7 +1056,7 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
     const bool self_here = sj >= kt && sj < kt + cnt;
     const int sc = self_here ? sj - kt : -1;
     f2 G0 = pk(0.f, 0.f), G1 = G0, G2 = G0, Z = G0;
-    unsigned long long mask = self_mask(sc, step, normal);
+    unsigned long long mask = self_mask(sc, step);
     int c = 4 * B.lane;
     // (cntp is a whole number of steps; two to an unrolled iteration)
     for (int m = 0; m < iters; m += kVjpUnroll,
@@ -1072,9 +1070,9 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
                            yl = ld4(&T.yl[c]), zl = ld4(&T.zl[c]),
                            lx = ld4(&T.lx[c]), ly = ld4(&T.ly[c]),
                            lz = ld4(&T.lz[c]);
-          pair_vjp_j2<false>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x,
+          pair_vjp_j2<kSafe, false>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x,
                              ly.x, lz.x, c, -1, e2, m3, G0, G1, G2, Z);
-          pair_vjp_j2<false>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y,
+          pair_vjp_j2<kSafe, false>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y,
                              ly.y, lz.y, c + 2, -1, e2, m3, G0, G1, G2, Z);
         }
       } else {
@@ -1085,9 +1083,9 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
                            yl = ld4(&T.yl[c]), zl = ld4(&T.zl[c]),
                            lx = ld4(&T.lx[c]), ly = ld4(&T.ly[c]),
                            lz = ld4(&T.lz[c]);
-          pair_vjp_j2<true>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x, ly.x,
+          pair_vjp_j2<true, true>(jj, xh.x, yh.x, zh.x, xl.x, yl.x, zl.x, lx.x, ly.x,
                             lz.x, c, sc, e2, m3, G0, G1, G2, Z);
-          pair_vjp_j2<true>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y, ly.y,
+          pair_vjp_j2<true, true>(jj, xh.y, yh.y, zh.y, xl.y, yl.y, zl.y, lx.y, ly.y,
                             lz.y, c + 2, sc, e2, m3, G0, G1, G2, Z);
         }
       }
@@ -1105,7 +1103,7 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
 // Replay force (mixed): a_i = sum_{j != i} m_j d_ij / s^3 for the active
 // bodies at the predicted positions, with the i side's work split, tiles
 // and packed pair loop; the sums are double-single per lane, FP64 after.
-template <bool kMask>
+template <bool kSafe, bool kMask>
 __device__ __forceinline__ void pair_force2(const f2 (&ii)[6], f2 xh, f2 yh,
                                             f2 zh, f2 m, f2 xl, f2 yl, f2 zl,
                                             int c, int self, f2 e2, f2& ax,
@@ -1116,7 +1114,7 @@ __device__ __forceinline__ void pair_force2(const f2 (&ii)[6], f2 xh, f2 yh,
   const f2 s2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
   float s0, s1;
   upk(s2, s0, s1);
-  float r0 = rsqrt_of<kMask>(s0), r1 = rsqrt_of<kMask>(s1);
+  float r0 = rsqrt_of<kSafe>(s0), r1 = rsqrt_of<kSafe>(s1);
   if (kMask) {
     if (c == self) r0 = 0.f;
     if (c + 1 == self) r1 = 0.f;
@@ -1128,6 +1126,7 @@ __device__ __forceinline__ void pair_force2(const f2 (&ii)[6], f2 xh, f2 yh,
   az = fma2(mr3, dz, az);
 }
 
+template <bool kSafe>
 __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
                                             VjpSmem& T0, VjpSm& sm) {
   const VjpSide& V = A.V.si;
@@ -1140,7 +1139,6 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
                     pk(il.x, il.x), pk(il.y, il.y), pk(il.z, il.z)};
   const f2 e2 = pk(A.eps2f, A.eps2f);
   const int step = 4 * V.tpt;
-  const bool normal = normal_eps2(A.eps2f);
   DS dacc[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   VjpTileI& T = T0.i;
   for (int jt = B.beg; jt < B.end; jt += kVjpTile) {
@@ -1161,7 +1159,7 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
     const bool self_here = B.live && bi >= jt && bi < jt + cnt;
     const int sc = self_here ? bi - jt : -1;
     f2 ax = pk(0.f, 0.f), ay = ax, az = ax;
-    unsigned long long mask = self_mask(sc, step, normal);
+    unsigned long long mask = self_mask(sc, step);
     int c = 4 * B.lane;
     // (cntp is a whole number of steps; two to an unrolled iteration)
     for (int m = 0; m < iters; m += kVjpUnroll,
@@ -1174,9 +1172,9 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
                            zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
                            xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
                            zl = ld4(&T.zl[c]);
-          pair_force2<false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, -1,
+          pair_force2<kSafe, false>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, -1,
                              e2, ax, ay, az);
-          pair_force2<false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+          pair_force2<kSafe, false>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
                              -1, e2, ax, ay, az);
         }
       } else {
@@ -1186,9 +1184,9 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
                            zh = ld4(&T.zh[c]), m = ld4(&T.m[c]),
                            xl = ld4(&T.xl[c]), yl = ld4(&T.yl[c]),
                            zl = ld4(&T.zl[c]);
-          pair_force2<true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
+          pair_force2<true, true>(ii, xh.x, yh.x, zh.x, m.x, xl.x, yl.x, zl.x, c, sc,
                             e2, ax, ay, az);
-          pair_force2<true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
+          pair_force2<true, true>(ii, xh.y, yh.y, zh.y, m.y, xl.y, yl.y, zl.y, c + 2,
                             sc, e2, ax, ay, az);
         }
       }
@@ -1203,14 +1201,15 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
   vjp_finish<2>(A, V, B, A.n_act, acc, A.O.part_i, A.O.cnt_i, sm);
 }
 
+template <bool kSafe>
 __global__ void __launch_bounds__(kAdjThreads, kVjpMinBlocks)
     adj_force_kernel(VjpArgs A) {
   __shared__ VjpSm sm;
   __shared__ VjpSmem tile;
-  force_mixed(A, blockIdx.x, tile, sm);
+  force_mixed<kSafe>(A, blockIdx.x, tile, sm);
 }
 
-template <int kMixed>
+template <int kMixed, bool kSafe>
 __global__ void __launch_bounds__(kAdjThreads, kVjpMinBlocks)
     adj_vjp_kernel(VjpArgs A) {
   const int b = blockIdx.x;
@@ -1218,9 +1217,9 @@ __global__ void __launch_bounds__(kAdjThreads, kVjpMinBlocks)
   if (kMixed) {
     __shared__ VjpSmem tile;
     if (b < A.iblocks)
-      vjp_i_mixed(A, b, tile, sm);
+      vjp_i_mixed<kSafe>(A, b, tile, sm);
     else
-      vjp_j_mixed(A, b - A.iblocks, tile, sm);
+      vjp_j_mixed<kSafe>(A, b - A.iblocks, tile, sm);
   } else {
     if (b < A.iblocks)
       vjp_i_f64(A, b, sm);
@@ -1456,7 +1455,9 @@ void launch_adj_force(int n, int n_act, const int* idx, double eps2,
   A.P = P;
   A.V.si = si;
   A.O = O;
-  adj_force_kernel<<<si.groups * si.S, kAdjThreads, 0, s>>>(A);
+  auto* k = normal_eps2(A.eps2f) ? adj_force_kernel<false>
+                                 : adj_force_kernel<true>;
+  k<<<si.groups * si.S, kAdjThreads, 0, s>>>(A);
 }
 
 void launch_adj_back_step(int n, double inv_ticks, int mixed,
@@ -1497,10 +1498,10 @@ void launch_adj_vjp(int mixed, int n, int n_act, const int* idx, double eps2,
   A.iblocks = V.si.groups * V.si.S;
   A.O = O;
   const int grid = A.iblocks + V.sj.groups * V.sj.S;
-  if (mixed)
-    adj_vjp_kernel<1><<<grid, kAdjThreads, 0, s>>>(A);
-  else
-    adj_vjp_kernel<0><<<grid, kAdjThreads, 0, s>>>(A);
+  auto* k = !mixed ? adj_vjp_kernel<0, false>
+            : normal_eps2(A.eps2f) ? adj_vjp_kernel<1, false>
+                                   : adj_vjp_kernel<1, true>;
+  k<<<grid, kAdjThreads, 0, s>>>(A);
 }
 
 void launch_adj_loss(int n, const double* m, const AdjState& St, double* out,

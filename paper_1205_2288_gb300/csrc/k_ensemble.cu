@@ -464,9 +464,9 @@ __device__ __forceinline__ void pair_mixed(const MixI& I,
 // so what the single-system item gains with two bodies per thread it would
 // lose to its longer prologue. In a full tile thread jl takes the j quads
 // 4 jl + 4 JG m. A body's own j is masked: the warp ORs the loop iterations
-// that hold one of its bodies, and only those (and all of them where eps^2
-// is no normal float) run the masked form, which rounds like the other one,
-// so a body's sums do not depend on its warp-mates. (With the whole tile
+// that hold one of its bodies, and only those run the masked form, which
+// rounds like the others (two: a cluster whose eps^2 is no normal float takes
+// rsqrtf), so a body's sums do not depend on its warp-mates. (With the whole tile
 // masked whenever one of 32 bodies lay in it, most tiles of a partial
 // active set ran masked.)
 template <int IG>
@@ -518,24 +518,29 @@ __device__ void ens_tiled_item(const ForceArgs& A, int n_act, const Plan& P,
       f2 p[4] = {z, z, z, z};
       const int self = valid && i >= jt && i < jt + cnt ? i - jt : -1;
       const int own = self < 0 ? -1 : self / (4 * JG);  // its iteration
-      unsigned long long mask = ~0ULL;
-      if (normal) {
-        const unsigned lo = __reduce_or_sync(
-            kFull, own >= 0 && own < 32 ? 1u << own : 0u);
-        unsigned hi = 0;
-        if (kIter > 32)
-          hi = __reduce_or_sync(kFull, own >= 32 ? 1u << (own - 32) : 0u);
-        mask = ((unsigned long long)hi << 32) | lo;
-      }
+      const unsigned lo =
+          __reduce_or_sync(kFull, own >= 0 && own < 32 ? 1u << own : 0u);
+      unsigned hi = 0;
+      if (kIter > 32)
+        hi = __reduce_or_sync(kFull, own >= 32 ? 1u << (own - 32) : 0u);
+      unsigned long long mask = ((unsigned long long)hi << 32) | lo;
       for (int m = 0; m < kIter; m += U, mask >>= U) {
         const int c0 = 4 * (jl + JG * m);
-        if ((mask & ((1ULL << U) - 1)) == 0) {
+        if ((mask & ((1ULL << U) - 1)) == 0 && normal) {
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             J2 a, b;
             load_j4(T, c0 + 4 * JG * u, a, b);
-            pair_mixed2<true, false>(ii, a, 0, e2, p, q);
-            pair_mixed2<true, false>(ii, b, 0, e2, p, q);
+            pair_mixed2<true, false, false>(ii, a, 0, e2, p, q);
+            pair_mixed2<true, false, false>(ii, b, 0, e2, p, q);
+          }
+        } else if ((mask & ((1ULL << U) - 1)) == 0) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            J2 a, b;
+            load_j4(T, c0 + 4 * JG * u, a, b);
+            pair_mixed2<true, true, false>(ii, a, 0, e2, p, q);
+            pair_mixed2<true, true, false>(ii, b, 0, e2, p, q);
           }
         } else {
 #pragma unroll 1
@@ -543,9 +548,8 @@ __device__ void ens_tiled_item(const ForceArgs& A, int n_act, const Plan& P,
             const int c = c0 + 4 * JG * u;
             J2 a, b;
             load_j4(T, c, a, b);
-            pair_mixed2<true, true>(ii, a, c, e2, p, q, self);
-            pair_mixed2<true, true>(ii, b, c + 2, e2, p, q,
-                                    self);
+            pair_mixed2<true, true, true>(ii, a, c, e2, p, q, self);
+            pair_mixed2<true, true, true>(ii, b, c + 2, e2, p, q, self);
           }
         }
       }

@@ -147,8 +147,9 @@ __global__ void __launch_bounds__(kThreads)
 
 // kPhi: the potential is summed (26 against 25 FMA-pipe operations; the
 // integrator does not read it). kSorted: bodies in spatial order, large
-// active sets by far_item.
-template <bool kPhi, bool kSorted>
+// active sets by far_item. kSafe: eps^2 is no normal float (never with
+// kSorted).
+template <bool kPhi, bool kSorted, bool kSafe>
 __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
     force_mixed_kernel(const __grid_constant__ ForceArgs A,
                        const __grid_constant__ PlanTable PT) {
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
   int n_act = 0;
   if (!force_prologue(A, n_act)) return;
   if constexpr (kSorted) {
-    if (n_act >= A.far_min && normal_eps2(A.eps2f)) {
+    if (n_act >= A.far_min) {
       FarSm& far = *reinterpret_cast<FarSm*>(smem);
       const int S = far_splits(n_act, A.n, gridDim.x, A.part_cap);
       if (blockIdx.x == 0 && threadIdx.x == 0 && A.nsplit_out)
@@ -196,12 +197,12 @@ __global__ void __launch_bounds__(kThreads, kMixMinBlocks)
   }
   MixTile<kTileMix>& T = *reinterpret_cast<MixTile<kTileMix>*>(smem);
   switch (P.ig) {
-    case 256: mixed_items<1, kPhi>(A, n_act, P, T); break;
-    case 128: mixed_items<2, kPhi>(A, n_act, P, T); break;
-    case 64: mixed_items<4, kPhi>(A, n_act, P, T); break;
-    case 32: mixed_items<8, kPhi>(A, n_act, P, T); break;
-    case 16: mixed_items<16, kPhi>(A, n_act, P, T); break;
-    default: mixed_items<32, kPhi>(A, n_act, P, T); break;
+    case 256: mixed_items<1, kPhi, kSafe>(A, n_act, P, T); break;
+    case 128: mixed_items<2, kPhi, kSafe>(A, n_act, P, T); break;
+    case 64: mixed_items<4, kPhi, kSafe>(A, n_act, P, T); break;
+    case 32: mixed_items<8, kPhi, kSafe>(A, n_act, P, T); break;
+    case 16: mixed_items<16, kPhi, kSafe>(A, n_act, P, T); break;
+    default: mixed_items<32, kPhi, kSafe>(A, n_act, P, T); break;
   }
 }
 
@@ -302,7 +303,7 @@ ForceLaunch force_launch_shape(int precision, int device) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (precision)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, force_mixed_kernel<true, false>, kThreads, 0);
+        &per_sm, force_mixed_kernel<true, false, false>, kThreads, 0);
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, force_fp64_kernel,
                                                   kThreads, 0);
@@ -340,10 +341,14 @@ cudaError_t launch_force(int precision, const ForceArgs& fa,
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   if (precision) {
-    auto* k = fa.no_phi ? (fa.meta ? force_mixed_kernel<false, true>
-                                   : force_mixed_kernel<false, false>)
-                        : (fa.meta ? force_mixed_kernel<true, true>
-                                   : force_mixed_kernel<true, false>);
+    auto* k = fa.no_phi ? force_mixed_kernel<false, false, false>
+                        : force_mixed_kernel<true, false, false>;
+    if (!normal_eps2(fa.eps2f))
+      k = fa.no_phi ? force_mixed_kernel<false, false, true>
+                    : force_mixed_kernel<true, false, true>;
+    else if (fa.meta)
+      k = fa.no_phi ? force_mixed_kernel<false, true, false>
+                    : force_mixed_kernel<true, true, false>;
     return cudaLaunchKernelEx(&cfg, k, fa, pt ? *pt : none);
   }
   if (fa.exact) {

@@ -182,6 +182,11 @@ struct Plan {
   int direct;
 };
 
+// eps^2 for which every s^2 is a normal float
+__host__ __device__ inline bool normal_eps2(float eps2) {
+  return eps2 >= 1.17549435e-38f;
+}
+
 // Arguments of the force kernels (shared by the integrator and the
 // stand-alone force entry point).
 struct ForceArgs {
