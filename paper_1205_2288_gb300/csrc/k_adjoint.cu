@@ -69,8 +69,6 @@ constexpr int kAdjThreads = 128;
 #endif
 constexpr int kVjpTpt = TSBTS_VJP_TPT;
 constexpr int kVjpSmax = TSBTS_VJP_SMAX;
-constexpr int kVjpFewGroups = 8;  // target groups that take more splits
-constexpr int kVjpSmaxFew = 64;
 constexpr int kVjpMinBlocks = TSBTS_VJP_MINB;
 constexpr int kVjpUnroll = TSBTS_VJP_UNROLL;
 
@@ -978,7 +976,7 @@ __device__ __forceinline__ void vjp_i_mixed(const VjpArgs& A, int b,
     f2 W = pk(0.f, 0.f), Ux = W, Uy = W, Uz = W;
     unsigned long long mask = self_mask(sc, step);
     int c = 4 * B.lane;
-    // (cntp is a whole number of steps; two to an unrolled iteration)
+    // (cntp is a whole number of steps; kVjpUnroll to an unrolled iteration)
     for (int m = 0; m < iters; m += kVjpUnroll,
              mask = (mask >> kVjpUnroll) | (mask << (64 - kVjpUnroll))) {
       if (m + kVjpUnroll <= iters &&
@@ -1058,7 +1056,7 @@ __device__ __forceinline__ void vjp_j_mixed(const VjpArgs& A, int b,
     f2 G0 = pk(0.f, 0.f), G1 = G0, G2 = G0, Z = G0;
     unsigned long long mask = self_mask(sc, step);
     int c = 4 * B.lane;
-    // (cntp is a whole number of steps; two to an unrolled iteration)
+    // (cntp is a whole number of steps; kVjpUnroll to an unrolled iteration)
     for (int m = 0; m < iters; m += kVjpUnroll,
              mask = (mask >> kVjpUnroll) | (mask << (64 - kVjpUnroll))) {
       if (m + kVjpUnroll <= iters &&
@@ -1161,7 +1159,7 @@ __device__ __forceinline__ void force_mixed(const VjpArgs& A, int b,
     f2 ax = pk(0.f, 0.f), ay = ax, az = ax;
     unsigned long long mask = self_mask(sc, step);
     int c = 4 * B.lane;
-    // (cntp is a whole number of steps; two to an unrolled iteration)
+    // (cntp is a whole number of steps; kVjpUnroll to an unrolled iteration)
     for (int m = 0; m < iters; m += kVjpUnroll,
              mask = (mask >> kVjpUnroll) | (mask << (64 - kVjpUnroll))) {
       if (m + kVjpUnroll <= iters &&
@@ -1330,14 +1328,16 @@ void set_splits(VjpSide& v, long long ns, long long S) {
   v.S = (int)std::max<long long>(1, (ns + chunk - 1) / chunk);
 }
 
-// split counts a side may take: at least one quad per lane for few target
-// groups, else 16 sources per lane
-int split_choices(const VjpSide& v, long long ns, int (&out)[17]) {
-  static const int kS[17] = {1,  2,  3,  4,  5,  6,  7,  8, 10,
-                             12, 14, 16, 20, 24, 32, 48, 64};
-  const bool few = v.groups <= kVjpFewGroups;
-  const long long cap = std::min<long long>(
-      few ? kVjpSmaxFew : kVjpSmax, ns / ((few ? 4LL : 16LL) * v.tpt));
+// Split counts a side may take: at least 16 sources per lane. (Few target
+// groups with down to one quad per lane, up to 64 splits, was faster by 4 to
+// 7% a step for up to three active bodies of 3000 and 8192, and slower by 7
+// to 20% for 10 to 100 of them and in systems of 300 and 500: gradients
+// 46.9 -> 45.4 ms at n = 8192, 14.5 -> 15.0 at 3000, 10.2 -> 11.1 at 500;
+// with this rule 44.5, 13.7, 9.94.)
+int split_choices(const VjpSide& v, long long ns, int (&out)[12]) {
+  static const int kS[12] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16};
+  static_assert(kVjpSmax <= 16, "split counts");
+  const long long cap = std::min<long long>(kVjpSmax, ns / (16LL * v.tpt));
   int m = 0;
   for (int S : kS)
     if (S == 1 || S <= cap) out[m++] = S;
@@ -1356,7 +1356,7 @@ constexpr double kVjpBlockCost = 32.0;
 
 void choose_splits(VjpSide& si, long long ns_i, VjpSide* sj, long long ns_j,
                    int sms) {
-  int ci[17], cj[17] = {1};
+  int ci[12], cj[12] = {1};
   const int mi = split_choices(si, ns_i, ci);
   const int mj = sj ? split_choices(*sj, ns_j, cj) : 1;
   double best = 1e300;
