@@ -844,7 +844,7 @@ int adjoint_init(tsbts_ctx* ctx, int64_t n, double eps, int64_t n_pass,
       grp_i = std::max<long long>(grp_i, v.si.groups);
       grp_j = std::max<long long>(grp_j, v.sj.groups);
     };
-    A.shape_init = vjp_shape(ni, ni, ctx->sms);
+    A.shape_init = vjp_shape(ni, ni, A.mixed, ctx->sms);
     need(A.shape_init);
     // (rated once per active count, as the plans below: a step's own rating
     // took 2 us, a third of the whole call for 3 x 1024 steps of 1000 bodies)
@@ -852,7 +852,7 @@ int adjoint_init(tsbts_ctx* ctx, int64_t n, double eps, int64_t n_pass,
     for (long long s = 0; s < A.S; ++s) {
       const int na = (int)(A.off[s + 1] - A.off[s]);
       A.shapes[s] = like[s] < s ? A.shapes[like[s]]
-                                : vjp_shape(ni, na, ctx->sms);
+                                : vjp_shape(ni, na, A.mixed, ctx->sms);
       need(A.shapes[s]);
     }
     A.O.part_i = adj_alloc<double>(A, cap_i);

@@ -1328,16 +1328,25 @@ void set_splits(VjpSide& v, long long ns, long long S) {
   v.S = (int)std::max<long long>(1, (ns + chunk - 1) / chunk);
 }
 
-// Split counts a side may take: at least 16 sources per lane. (Few target
-// groups with down to one quad per lane, up to 64 splits, was faster by 4 to
-// 7% a step for up to three active bodies of 3000 and 8192, and slower by 7
-// to 20% for 10 to 100 of them and in systems of 300 and 500: gradients
-// 46.9 -> 45.4 ms at n = 8192, 14.5 -> 15.0 at 3000, 10.2 -> 11.1 at 500;
-// with this rule 44.5, 13.7, 9.94.)
-int split_choices(const VjpSide& v, long long ns, int (&out)[12]) {
-  static const int kS[12] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16};
-  static_assert(kVjpSmax <= 16, "split counts");
-  const long long cap = std::min<long long>(kVjpSmax, ns / (16LL * v.tpt));
+// Split counts a side may take. Mixed: at least 16 sources per lane. (Few
+// target groups with down to one quad per lane, up to 64 splits, was faster
+// by 4 to 7% a step for up to three active bodies of 3000 and 8192, and
+// slower by 7 to 20% for 10 to 100 of them and in systems of 300 and 500:
+// gradients 46.9 -> 45.4 ms at n = 8192, 14.5 -> 15.0 at 3000, 10.2 -> 11.1
+// at 500; with this rule 44.5, 13.7, 9.94.) FP64: up to kVjpFewGroups target
+// groups (128 active bodies at four lanes each and half the grid's SMs idle)
+// go down to four sources per lane, each of which costs some 50 FP64
+// instructions of 64 cycles: gradients 30.4 -> 25.7 ms at n = 600, a step on
+// 30 of 9000 bodies 389 -> 281 us, on 300 and more the same.
+constexpr int kVjpFewGroups = 8;
+constexpr int kVjpSmaxFew = 64;
+
+int split_choices(const VjpSide& v, long long ns, int mixed, int (&out)[17]) {
+  static const int kS[17] = {1,  2,  3,  4,  5,  6,  7,  8, 10,
+                             12, 14, 16, 20, 24, 32, 48, 64};
+  const bool few = !mixed && v.groups <= kVjpFewGroups;
+  const long long cap = std::min<long long>(
+      few ? kVjpSmaxFew : kVjpSmax, ns / ((few ? 4LL : 16LL) * v.tpt));
   int m = 0;
   for (int S : kS)
     if (S == 1 || S <= cap) out[m++] = S;
@@ -1355,10 +1364,10 @@ constexpr int kVjpResident = 4;
 constexpr double kVjpBlockCost = 32.0;
 
 void choose_splits(VjpSide& si, long long ns_i, VjpSide* sj, long long ns_j,
-                   int sms) {
-  int ci[12], cj[12] = {1};
-  const int mi = split_choices(si, ns_i, ci);
-  const int mj = sj ? split_choices(*sj, ns_j, cj) : 1;
+                   int mixed, int sms) {
+  int ci[17], cj[17] = {1};
+  const int mi = split_choices(si, ns_i, mixed, ci);
+  const int mj = sj ? split_choices(*sj, ns_j, mixed, cj) : 1;
   double best = 1e300;
   int bi = 1, bj = 1;
   for (int x = 0; x < mi; ++x)
@@ -1391,13 +1400,13 @@ void choose_splits(VjpSide& si, long long ns_i, VjpSide* sj, long long ns_j,
 
 }  // namespace
 
-VjpShape vjp_shape(int n, int n_act, int sms) {
+VjpShape vjp_shape(int n, int n_act, int mixed, int sms) {
   VjpShape s;
   s.si = side_of(n_act, n);
   s.sf = s.si;
   s.sj = side_of(n, n_act);
-  choose_splits(s.si, n, &s.sj, n_act, sms);
-  choose_splits(s.sf, n, nullptr, 0, sms);
+  choose_splits(s.si, n, &s.sj, n_act, mixed, sms);
+  choose_splits(s.sf, n, nullptr, 0, mixed, sms);
   return s;
 }
 

@@ -126,7 +126,7 @@ struct VjpSide {
 struct VjpShape {
   VjpSide si, sj, sf;
 };
-VjpShape vjp_shape(int n, int n_act, int sms);
+VjpShape vjp_shape(int n, int n_act, int mixed, int sms);
 // results of one force vector-Jacobian product: u[3] per active slot (i
 // side) and G[3], Z per body in g[4] (j side); split partials and the
 // per-group completion counters (zero between launches)
