@@ -5,9 +5,9 @@
 // small boxes. Most pairs of a warp and a subtile are then far apart, and
 // far pairs need less work for the same result:
 //  - coordinates: x'_j = x_j - c and x'_i = x_i - c, each rounded once to
-//    FP32 about the centre c of the block's 256 bodies, leave one
-//    subtraction per component instead of the three of the double-single
-//    difference. Where the boxes are further apart than the radius rho of
+//    FP32 about the centre c of the block's 256 bodies (far_rule.h: once per
+//    staged j, 3 of 250 additions a pair), leave one subtraction per
+//    component instead of the three of the double-single difference. Where the boxes are further apart than the radius rho of
 //    those bodies, |x'_j| + |x'_i| <= 3 |d|, so the rounding of x'_j and
 //    x'_i is at most 3/2 units of d's last place, as the two roundings of the
 //    double-single difference of far bodies are one;
@@ -25,6 +25,7 @@
 // 2-norms): a 2.7e-8 (3.2e-8 unsorted), phi 7e-9 (9e-9), q 1.1e-7 (1.1e-7).
 #pragma once
 
+#include "far_rule.h"
 #include "force_device.cuh"
 
 namespace tsbts {
@@ -250,7 +251,7 @@ __device__ __forceinline__ void far_item(const ForceArgs& A, int n_act, int g,
     for (int c = 0; c < 9; ++c) ii[r][c] = pk(x[c], x[c]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float d = (x[c] - cen[c]) + x[3 + c];
+      const float d = about(x[c], x[3 + c], cen[c]);
       ci[r][c] = pk(d, d);
     }
   }
@@ -273,9 +274,9 @@ __device__ __forceinline__ void far_item(const ForceArgs& A, int n_act, int g,
       T.t.xh[c] = h.x; T.t.yh[c] = h.y; T.t.zh[c] = h.z; T.t.m[c] = h.w;
       T.t.xl[c] = l.x; T.t.yl[c] = l.y; T.t.zl[c] = l.z;
       T.t.u[c] = v.x; T.t.v[c] = v.y; T.t.w[c] = v.z;
-      T.cx[c] = (h.x - cen[0]) + l.x;
-      T.cy[c] = (h.y - cen[1]) + l.y;
-      T.cz[c] = (h.z - cen[2]) + l.z;
+      T.cx[c] = about(h.x, l.x, cen[0]);
+      T.cy[c] = about(h.y, l.y, cen[1]);
+      T.cz[c] = about(h.z, l.z, cen[2]);
     }
     __syncthreads();
     // the tile's subtiles as this warp sees them (lane e: subtile e)
