@@ -501,7 +501,7 @@ void setup_bodies(tsbts_ctx* c, int n, bool sorted) {
     B.amask = dalloc<unsigned>(L, words);
     B.meta = dalloc<float4>(L, 2 * words);
     c->sort_key = dalloc<unsigned long long>(L, sort_capacity(n));
-    c->d_sort = dalloc<double>(L, 128);
+    c->d_sort = dalloc<double>(L, kSortPart);
   }
   Bodies& S = c->snap;
   S = Bodies{};
@@ -753,7 +753,7 @@ struct Scratch {
   int* nsplit = nullptr;
   int* iota = nullptr;    // 0, 1, ..., n_cap - 1 (active list for tuning)
   // spatial order (calls that sort): order, slot, list and pos in `sort_i`
-  // (4 n_cap), keys, subtile summaries, 128 doubles
+  // (4 n_cap), keys, subtile summaries, kSortPart doubles
   int* sort_i = nullptr;
   unsigned long long* key = nullptr;
   float4* meta = nullptr;
@@ -1319,7 +1319,7 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
            "scratch");
         ck(cudaMalloc(&S.meta, sizeof(float4) * 2 * (cap / 32 + 1)),
            "scratch");
-        ck(cudaMalloc(&S.scale, sizeof(double) * 128), "scratch");
+        ck(cudaMalloc(&S.scale, sizeof(double) * kSortPart), "scratch");
         S.sort_cap = (int)cap;
         S.sort_stride = cap;
       }

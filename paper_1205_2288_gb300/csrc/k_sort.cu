@@ -1,7 +1,9 @@
 // Spatial order of bodies for the mixed force (force_far.cuh): positions along
-// a Hilbert curve and a bitonic sort of 64-bit keys (curve position above,
-// index below, so the order is unique and the same on every run). The sort runs once per era (or force call) on at most 2^20 keys;
-// its launches, not its work, are its cost (about 30 at 2^17 keys).
+// a Hilbert curve (far_rule.h) and a bitonic sort of 64-bit keys (curve
+// position above, index below, so the order is unique and the same on every
+// run). The sort runs once per era (or force call) on at most 2^20 keys; its
+// launches, not its work, are its cost (about 30 at 2^17 keys).
+#include "far_rule.h"
 #include "tsbts_kernels.cuh"
 
 namespace tsbts {
@@ -11,15 +13,58 @@ namespace {
 constexpr int kSortThreads = 1024;
 constexpr int kSortLocal = 2 * kSortThreads;  // keys sorted in shared memory
 constexpr int kScaleBlocks = 128;
+static_assert(kScaleBlocks + 3 == kSortPart, "partial sums and centre");
+
+__device__ __forceinline__ void exchange(unsigned long long& a,
+                                         unsigned long long& b, bool up) {
+  if ((a > b) == up) {
+    const unsigned long long t = a;
+    a = b;
+    b = t;
+  }
+}
+
+// the bodies' centre, into part[kScaleBlocks ..]: block a takes the median of
+// coordinate a over a sample, by a bitonic sort of the bit patterns
+__global__ void __launch_bounds__(kCentreSample)
+    sort_centre_kernel(int n, const double* x, const double* y,
+                       const double* z, int stride, double* part) {
+  __shared__ unsigned long long s[kCentreSample];
+  const double* p = blockIdx.x == 0 ? x : (blockIdx.x == 1 ? y : z);
+  const int t = threadIdx.x, m = min(n, kCentreSample);
+  unsigned long long u = ~0ULL;
+  if (t < m) {
+    const int i = n > kCentreSample ? centre_sample(t, n) : t;
+    u = (unsigned long long)__double_as_longlong(p[(long long)i * stride]);
+    u = u >> 63 ? ~u : u | 1ULL << 63;  // ordered like the doubles
+  }
+  s[t] = u;
+  for (int k = 2; k <= kCentreSample; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      __syncthreads();
+      const int o = t ^ j;
+      if (o > t) exchange(s[t], s[o], (t & k) == 0);
+    }
+  __syncthreads();
+  if (t == 0) {
+    u = s[m / 2];
+    const double c =
+        __longlong_as_double((long long)(u >> 63 ? u & ~(1ULL << 63) : ~u));
+    part[kScaleBlocks + blockIdx.x] = isfinite(c) ? c : 0.0;
+  }
+}
 
 __global__ void __launch_bounds__(256)
     sort_scale_kernel(int n, const double* x, const double* y,
                       const double* z, int stride, double* part) {
   __shared__ float sm[256];
+  const double cx = part[kScaleBlocks], cy = part[kScaleBlocks + 1],
+               cz = part[kScaleBlocks + 2];
   float s = 0.f;
   for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += kScaleBlocks * 256) {
     const long long o = (long long)i * stride;
-    s += fabsf((float)x[o]) + fabsf((float)y[o]) + fabsf((float)z[o]);
+    s += fabsf((float)(x[o] - cx)) + fabsf((float)(y[o] - cy)) +
+         fabsf((float)(z[o] - cz));
   }
   sm[threadIdx.x] = s;
   __syncthreads();
@@ -28,47 +73,6 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
   }
   if (threadIdx.x == 0) part[blockIdx.x] = (double)sm[0];
-}
-
-// 10 bits of a coordinate, mapped to (-1, 1) by x / (|x| + scale)
-__device__ __forceinline__ unsigned cell(float x, float scale) {
-  const float u = x / (fabsf(x) + scale);
-  return (unsigned)min(1023, max(0, (int)((u * 0.5f + 0.5f) * 1024.f)));
-}
-
-// Position along the Hilbert curve of a cell (10 bits per axis), by
-// J. Skilling's transform ("Programming the Hilbert curve", AIP Conf. Proc.
-// 707, 2004): undo the excess work from the top bit down, Gray-encode,
-// interleave. Runs of consecutive bodies fill smaller boxes than in Morton
-// order, whose jumps leave 47% of the subtiles of 131072 bodies too near for
-// the cheap form, against 25%.
-__device__ __forceinline__ unsigned hilbert(unsigned x, unsigned y,
-                                            unsigned z) {
-  unsigned X[3] = {x, y, z};
-  for (unsigned Q = 512; Q > 1; Q >>= 1) {
-    const unsigned P = Q - 1;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      if (X[i] & Q) {
-        X[0] ^= P;
-      } else {
-        const unsigned t = (X[0] ^ X[i]) & P;
-        X[0] ^= t;
-        X[i] ^= t;
-      }
-    }
-  }
-  X[1] ^= X[0];
-  X[2] ^= X[1];
-  unsigned t = 0;
-  for (unsigned Q = 512; Q > 1; Q >>= 1)
-    if (X[2] & Q) t ^= Q - 1;
-  unsigned h = 0;
-#pragma unroll
-  for (int b = 9; b >= 0; --b)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) h = h << 1 | ((X[i] ^ t) >> b & 1u);
-  return h;
 }
 
 __global__ void __launch_bounds__(256)
@@ -89,21 +93,13 @@ __global__ void __launch_bounds__(256)
   unsigned long long k = ~0ULL;
   if (i < n) {
     const long long o = (long long)i * stride;
-    const unsigned m = hilbert(cell((float)x[o], scale),
-                               cell((float)y[o], scale),
-                               cell((float)z[o], scale));
+    const double* c = part + kScaleBlocks;
+    const unsigned m = hilbert(curve_cell((float)(x[o] - c[0]), scale),
+                               curve_cell((float)(y[o] - c[1]), scale),
+                               curve_cell((float)(z[o] - c[2]), scale));
     k = (unsigned long long)m << 32 | (unsigned)i;
   }
   key[i] = k;
-}
-
-__device__ __forceinline__ void exchange(unsigned long long& a,
-                                         unsigned long long& b, bool up) {
-  if ((a > b) == up) {
-    const unsigned long long t = a;
-    a = b;
-    b = t;
-  }
 }
 
 // strides j_first .. 1 of the merge of size k (k0 .. k1), inside blocks of
@@ -189,12 +185,13 @@ int launch_spatial_order(int n, const double* x, const double* y,
                          unsigned long long* key, int* order, int* slot,
                          cudaStream_t s) {
   const int n2 = sort_capacity(n);
+  sort_centre_kernel<<<3, kCentreSample, 0, s>>>(n, x, y, z, stride, part);
   sort_scale_kernel<<<kScaleBlocks, 256, 0, s>>>(n, x, y, z, stride, part);
   sort_keys_kernel<<<blocks(n2), 256, 0, s>>>(n, n2, x, y, z, stride, part,
                                               key);
   const int l = sort_keys(key, n2, s);
   order_kernel<<<blocks(n), 256, 0, s>>>(n, key, order, slot);
-  return l + 3;
+  return l + 4;
 }
 
 void launch_sorted_list(int n_act, const int* idx, const int* slot,

@@ -436,8 +436,9 @@ cudaError_t launch_force_finalize(const double* part, int S, int n_act,
                                   const int* pos, double* a, double* phi,
                                   double* q, cudaStream_t s);
 // spatial order (k_sort.cu): keys a sort of n needs; order (and its inverse
-// slot, nullable) of bodies with coordinates x[i * stride] ...; part: 128
-// doubles; returns the number of launches
+// slot, nullable) of bodies with coordinates x[i * stride] ...; part:
+// kSortPart doubles; returns the number of launches
+constexpr int kSortPart = 131;
 int sort_capacity(long long n);
 int launch_spatial_order(int n, const double* x, const double* y,
                          const double* z, int stride, double* part,

@@ -6,7 +6,12 @@ their last place from the exact difference (plus what the two parts of x leave
 out, 2^-48 of x), and their errors have no mean beyond what so many uniform
 errors leave (five standard deviations of 0.29 units / sqrt(count)), with x's
 upper part cut toward zero as the integrator cuts it, and rounded as the force
-call does."""
+call does.
+
+The curve's cells are the bodies' own: a Plummer sphere that was moved has as
+many far pairs of a warp's bodies and a subtile as one about the coordinate
+origin (within a tenth; the cells' edges lie elsewhere), also with a body far
+outside."""
 import ctypes as C
 import os
 import shutil
@@ -26,6 +31,17 @@ extern "C" void about_n(long long n, const float* h, const float* l, float c,
                         float* out) {
   for (long long i = 0; i < n; ++i) out[i] = tsbts::about(h[i], l[i], c);
 }
+extern "C" void sample_n(int n, int* out) {
+  for (int k = 0; k < tsbts::kCentreSample; ++k)
+    out[k] = tsbts::centre_sample(k, n);
+}
+extern "C" void keys_n(long long n, const float* x, float scale,
+                       unsigned* out) {
+  for (long long i = 0; i < n; ++i)
+    out[i] = tsbts::hilbert(tsbts::curve_cell(x[3 * i], scale),
+                            tsbts::curve_cell(x[3 * i + 1], scale),
+                            tsbts::curve_cell(x[3 * i + 2], scale));
+}
 """
 
 FP = C.POINTER(C.c_float)
@@ -43,6 +59,8 @@ def lib(tmp_path_factory):
                     str(src), "-o", str(so)], check=True)
     L = C.CDLL(str(so))
     L.about_n.argtypes = [C.c_longlong, FP, FP, C.c_float, FP]
+    L.sample_n.argtypes = [C.c_int, C.POINTER(C.c_int)]
+    L.keys_n.argtypes = [C.c_longlong, FP, C.c_float, C.POINTER(C.c_uint32)]
     return L
 
 
@@ -77,3 +95,42 @@ def test_one_rounding(lib, cut, c, shift):
             2.0 ** -48 * np.abs(x)).all()
     toward = (err / unit) * np.sign(x)
     assert abs(toward.mean()) < 5 * 0.29 / np.sqrt(len(x))
+
+
+def spatial_order(lib, r):
+    """Bodies along the curve, as launch_spatial_order lists them."""
+    n = len(r)
+    pick = np.empty(1024, np.int32)
+    lib.sample_n(n, pick.ctypes.data_as(C.POINTER(C.c_int)))
+    assert (np.diff(pick) > 0).all() and pick[0] >= 0 and pick[-1] < n
+    x = np.ascontiguousarray((r - np.sort(r[pick], 0)[512]), np.float32)
+    scale = 0.5 * np.abs(x).sum() / n
+    key = np.empty(n, np.uint32)
+    lib.keys_n(n, x.ctypes.data_as(FP), scale,
+               key.ctypes.data_as(C.POINTER(C.c_uint32)))
+    return np.lexsort((np.arange(n), key))
+
+
+def far_fraction(r, order):
+    """Pairs of a warp's 64 bodies and a subtile of 32 that are further apart
+    than the radius of the block's 256 bodies (all bodies active)."""
+    x = r[order][:len(r) // 256 * 256]
+    box = [(f(x.reshape(-1, k, 3), 1)) for k in (32, 64, 256)
+           for f in (np.min, np.max)]
+    jl, jh, wl, wh, bl, bh = box
+    rho2 = np.repeat(((bh - bl) ** 2).sum(1) / 4, 4)
+    far = 0
+    for w in range(0, len(wl), 8):
+        gap = np.maximum(0, np.maximum(jl - wh[w], wl[w] - jh))
+        far += ((gap ** 2).sum(1) > rho2[w]).mean()
+    return far / len(range(0, len(wl), 8))
+
+
+@pytest.mark.parametrize("shift", [10.0, 100.0, 3000.0, 1e6])
+def test_order_does_not_depend_on_the_origin(lib, shift):
+    r = inputs.plummer(65536, 3)[1]
+    r[77] = [1e5, -3e4, 2e4]
+    want = far_fraction(r, spatial_order(lib, r))
+    moved = r + shift * np.array([1.0, -0.6, 0.3])
+    got = far_fraction(moved, spatial_order(lib, moved))
+    assert want > 0.4 and got > 0.9 * want, (want, got)
