@@ -815,15 +815,18 @@ void free_sort(Scratch& S) {
   S.sort_stride = 0;
 }
 
-// Whether a mixed force call sorts its bodies: the sorts of the bodies and of
-// the active list take about 0.2 ms together, what far pairs save is about
-// a third of the time (2^31 interactions: 1.9 ms), and the active bodies
-// have to be dense enough for 256 of them to fill a small box.
+// Whether a mixed force call sorts its bodies. The sorts of the bodies and of
+// the active list take about 0.25 ms together, and the active bodies have to
+// be dense enough for 256 of them to fill a small box. Sorted and unsorted,
+// in ms: all of 46400 1.96 and 1.83, half of 65536 1.95 and 1.85, all of
+// them 3.33 and 3.68, half of 92000 3.62 and 3.61, all 6.02 and 7.21; an
+// eighth of 131072 2.14 and 1.86, a quarter 3.68 and 3.68, half 6.18 and
+// 7.33, all 11.25 and 14.67. Hence 2^32 interactions and a quarter.
 bool force_sorts(int precision, int64_t n, int64_t n_act, double eps) {
   const float eps2 = (float)(eps * eps);
   return precision == TSBTS_MIXED && n >= kSortMinBodies &&
-         n <= kSortMaxBodies && n_act >= n / kFarMinShare &&
-         n_act <= kSortMaxBodies && n * n_act >= (1LL << 31) &&
+         n <= kSortMaxBodies && n_act >= n / kSortMinShare &&
+         n_act <= kSortMaxBodies && n * n_act >= (1LL << 32) &&
          normal_eps2(eps2);
 }
 std::mutex g_scratch_mu;

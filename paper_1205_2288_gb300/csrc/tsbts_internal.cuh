@@ -225,14 +225,17 @@ struct ForceArgs {
 };
 
 // Bodies from which the mixed force keeps spatial order (integrator: sorted
-// once per era) or sorts (stand-alone call), and the fewest active ones, per
-// body, that take the far form. Below, reading the bodies through the order
-// in every prediction costs what the far pairs of large steps save: eras
-// against the unsorted force, 16384 bodies 109 and 98 ms, 25000 34.3 and
-// 31.5, 50000 84 and 98, 131072 269 and 389.
+// once per era) or may sort (stand-alone call, engine.cu), and the fewest
+// active ones, per body, that take the far form in the integrator and let a
+// call sort. Below, reading the bodies through the order in every prediction
+// costs what the far pairs of large steps save. Starts of eras in order and
+// unsorted, in ms: 16384 bodies 109 and 98, 25000 34.3 and 31.5, 32768 37.7
+// and 36.7, 36000 42.9 and 43.1, 45000 62.6 and 68.8, 65536 60.2 and 74.3,
+// 131072 271 and 389 (the unsorted form of then).
 constexpr int kSortMinBodies = 32768;
 constexpr int kSortMaxBodies = 1 << 20;
 constexpr int kFarMinShare = 16;
+constexpr int kSortMinShare = 4;
 
 // Measured work plans of the integrator's force launch, one per power-of-two
 // bucket of active counts (bucket b holds counts in (2^(b-1), 2^b], the last
