@@ -1313,7 +1313,8 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
                     cudaMemcpyHostToDevice),
          "scratch");
       if (ncap >= kSortMinBodies) {
-        // with the rest, so that no later call of this size allocates
+        // with the rest, whatever the precision (2% of it), so that no later
+        // call of this size allocates, which it could not under capture
         const size_t cap = (size_t)std::min<int64_t>(
             std::max<int64_t>(ncap, n_act), kSortMaxBodies);
         ck(cudaMalloc(&S.sort_i, sizeof(int) * 4 * cap), "scratch");
@@ -1398,7 +1399,10 @@ int tsbts_force(int precision, int exact_order, int64_t n, const double* m,
       fa.plan.S = far_splits_host((int)n_act, ni, fl.grid, S.part_cap);
     }
     fa.has_plan = 1;
-    if (std::getenv("TSBTS_PRINT_PLANS"))
+    if (std::getenv("TSBTS_PRINT_PLANS") && sorts)
+      std::fprintf(stderr, "tsbts_force n=%d n_act=%lld: spatial order, "
+                   "groups of 256, S %d\n", ni, (long long)n_act, fa.plan.S);
+    else if (std::getenv("TSBTS_PRINT_PLANS"))
       std::fprintf(stderr, "tsbts_force n=%d n_act=%lld: ig %d n_g %d S %d "
                    "chunk %d %s\n", ni, (long long)n_act, fa.plan.ig,
                    fa.plan.n_g, fa.plan.S, fa.plan.chunk,

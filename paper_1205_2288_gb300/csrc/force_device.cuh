@@ -15,8 +15,14 @@ constexpr int kTileMix = 512;   // j per shared-memory tile, mixed
 constexpr int kStrip = 256;     // j per thread between two folds, mixed
 constexpr int kLaneMinMix = 16; // fewest j per thread in a split item
 constexpr int kLaneMinF64 = 8;
-constexpr int kSplitCap = 16;   // most j-splits of one of many active bodies
-constexpr int kSplitCapFew = 64;  // ... of one of at most kFewBodies
+// Most j-splits of a tiled plan: kSplitCap, which bounds what the consumer
+// reads of many bodies, and kSplitCapFew for at most kFewBodies active ones,
+// whose groups leave SMs idle with 16. Of 131072 bodies, in us with 16 and
+// with 64: 64 active 47.4 and 32.0, 128 69.9 and 39.3, 256 64.6 and 53.6, 512
+// 94.6 and 82.3 (513, with 16: 98.9); of 20000 128 24.8 and 18.8, 512 27.0
+// and 25.7.
+constexpr int kSplitCap = 16;
+constexpr int kSplitCapFew = 64;
 constexpr int kFewBodies = 512;
 constexpr int kSplitCapDirect = 128;  // most j-splits of a direct-load plan
 constexpr int kDirectBatch = 4;  // j records per lane loaded in one batch

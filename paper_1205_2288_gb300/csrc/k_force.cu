@@ -72,7 +72,9 @@ Plan plan_force(int precision, int exact, int n_act, int n,
 // The plan of a launch: fixed by the caller or from the bucket table. A
 // bucket's plan was made for the bucket's largest count; a smaller count has
 // fewer groups, so its split count is chosen again (tiled: tiled_plan;
-// direct and FP64: as many as keep the grid full).
+// direct: as many as keep the grid full). FP64 keeps the bucket's split
+// count: where that fills the grid's two blocks per SM, half the groups still
+// give every SM one, which fills its FP64 pipe.
 __device__ __forceinline__ Plan launch_plan(const ForceArgs& A,
                                             const PlanTable& PT, int n_act,
                                             int precision) {
