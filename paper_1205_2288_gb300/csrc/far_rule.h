@@ -2,6 +2,8 @@
 // that host code can run too.
 #pragma once
 
+#include <cstring>
+
 #ifdef __CUDACC__
 #define TSBTS_HD __host__ __device__ __forceinline__
 #else
@@ -13,18 +15,53 @@ namespace tsbts {
 // x - c for x = h + l (|l| at most a unit in h's last place), rounded once:
 // the remainder of h - c is exact (Knuth's two-sum) and joins l before the
 // last addition. Rounded twice, as (h - c) + l, the result can be a whole
-// unit off instead of half of one, and it leans: h is cut toward zero in the
-// integrator, so that l has the sign of x, and it vanishes wherever h - c is
-// on a coarser grid than l. The mean error of a far pair's distance was
-// -9.8e-9 of it, and less than 1e-10 now (double-single form: -3.3e-9); the
-// energy of 36864 bodies after an era of 1/8 was 5.5e-11 of it off the FP64
-// path's with the same block steps, and 1.0e-11 now (unsorted form 0.2e-11,
-// the scheme's own error 1.9e-10).
+// unit off instead of half of one, and where h is cut toward zero it leans: l
+// has the sign of x, and it vanishes wherever h - c is on a coarser grid than
+// l. The mean error of a far pair's distance was then
+// -9.8e-9 of it, and is less than 1e-10 now; the energy of 36864 bodies after
+// an era of 1/8 was 5.5e-11 of it off the FP64 path's with the same block
+// steps, and 1.0e-11 with one rounding (see split_round for the rest).
 TSBTS_HD float about(float h, float l, float c) {
   const float t = h - c;
   const float b = t + c, a = t - b;
   const float e = (h - b) - (c + a);
   return t + (l + e);
+}
+
+// The bit pattern of one type as another of its size
+template <class To, class From>
+TSBTS_HD To bits_as(From x) {
+  static_assert(sizeof(To) == sizeof(From), "same size");
+  To y;
+  memcpy(&y, &x, sizeof y);
+  return y;
+}
+
+// Double-single split of x with hi rounded to nearest (ties away from zero)
+// and lo the exact remainder rounded to float, with integer operations and
+// one float product (the FP64 pipe, which the conversions would take, is 64
+// times narrower). For |x| in 2^-70 .. 2^100 (the caller's range test);
+// hi + lo is x to 2^-49.
+//
+// Rounded, not cut: the differences of a near pair, (h_j - h_i) + (l_j -
+// l_i), round the first part, and where that drops l_j - l_i, parts cut
+// toward zero leave the distance too short (3.3e-9 of it on average for
+// distant pairs of a Plummer sphere; rounded ones do not lean). Far pairs
+// have no such mean, and a pair's force changes by twice that difference
+// whenever it crosses between the two forms: the energy of 131072 bodies
+// after an era of 1/8 time units was 2.9e-11 of it off the unsorted form's
+// with cut parts, 0.4e-11 with rounded ones.
+TSBTS_HD void split_round(double x, float& hi, float& lo) {
+  const unsigned long long b = bits_as<unsigned long long>(x);
+  const int e = (int)((b >> 52) & 0x7ff);
+  const unsigned sign = (unsigned)(b >> 63) << 31;
+  const unsigned long long m = (b & ((1ULL << 52) - 1)) + (1ULL << 28);
+  // (a carry out of the significand goes into the exponent)
+  hi = bits_as<float>(sign | (((unsigned)(e - 1023 + 127) << 23) +
+                              (unsigned)(m >> 29)));
+  const int r = (int)(m & ((1u << 29) - 1)) - (1 << 28);
+  const float scale = bits_as<float>((unsigned)(e - 1023 - 52 + 127) << 23);
+  lo = bits_as<float>(bits_as<unsigned>((float)r * scale) ^ sign);
 }
 
 // Cells of the curve: 10 bits of a coordinate about the bodies' centre, mapped

@@ -173,7 +173,7 @@ __global__ void ens_predict_kernel(Bodies B, Params P, Ens E, History prev) {
       const long long nt = tj + dtj;
       act = (nt == tn);
       if (nt < tn) atomicOr(&ctl->err, kErrInvariant);
-      predict_body(B, P, prev, j, j, tj, tn, pass, act, L);
+      predict_body<false>(B, P, prev, j, j, tj, tn, pass, act, L);
     }
   }
   // lanes of one cluster share one atomic on the cluster's counter

@@ -137,7 +137,7 @@ __global__ void select_predict_kernel(Bodies B, Params P, History HA,
     const long long nt = tj + dtj;
     act = (nt == tn);
     if (nt < tn) atomicOr(&ctl->err, kErrInvariant);
-    predict_body(B, P, prev, j, slot, tj, tn, pass, act, L);
+    predict_body<kSorted>(B, P, prev, j, slot, tj, tn, pass, act, L);
   }
   // compaction of the active list (order within a step is arbitrary; in
   // spatial order a force launch on many bodies lists them by the masks)
@@ -530,7 +530,7 @@ __global__ void init_jdata_kernel(Bodies B, Params P) {
       rp[c] = B.r[c][j];
       vp[c] = B.v[c][j];
     }
-    store_prediction(B, P, j, j, rp, vp);
+    store_prediction<false>(B, P, j, j, rp, vp);
   }
 }
 

@@ -7,6 +7,7 @@
 
 #include <climits>
 
+#include "far_rule.h"
 #include "tsbts_internal.cuh"
 
 namespace tsbts {
@@ -16,13 +17,19 @@ namespace tsbts {
 // much as an FP64 add): hi is x with its significand cut to the leading 24
 // bits, lo the exact remainder rounded to float, so hi + lo equals x to
 // about 2^-48 relative. Doubles outside 2^-70 .. 2^100 in magnitude (and
-// zeros, non-finite values) take the conversion path.
+// zeros, non-finite values) take the conversion path. kRound (spatially
+// ordered runs): hi rounded to nearest (split_round).
+template <bool kRound>
 __device__ __forceinline__ void split_ds(double x, float& hi, float& lo) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
   if (e < 1023 - 70 || e > 1023 + 100) {
     hi = __double2float_rn(x);
     lo = __double2float_rn(x - (double)hi);
+    return;
+  }
+  if constexpr (kRound) {
+    split_round(x, hi, lo);
     return;
   }
   const unsigned sign = (unsigned)(b >> 63) << 31;
@@ -51,6 +58,7 @@ __device__ __forceinline__ float to_float(double x) {
 
 // j data of the force kernels at the block time: FP64 arrays or the packed
 // double-single records of the mixed path (body j's at index slot)
+template <bool kRound>
 __device__ __forceinline__ void store_prediction(const Bodies& B,
                                                  const Params& P, int j,
                                                  int slot,
@@ -63,7 +71,7 @@ __device__ __forceinline__ void store_prediction(const Bodies& B,
     }
   } else {
     float h[3], l[3];
-    for (int c = 0; c < 3; ++c) split_ds(rp[c], h[c], l[c]);
+    for (int c = 0; c < 3; ++c) split_ds<kRound>(rp[c], h[c], l[c]);
     B.jhi[slot] = make_float4(h[0], h[1], h[2], B.mf[j]);
     B.jlo[slot] = make_float4(l[0], l[1], l[2], 0.f);
     B.jv[slot] = make_float4(to_float(vp[0]), to_float(vp[1]), to_float(vp[2]),
@@ -118,6 +126,7 @@ __device__ __forceinline__ void load_pred_in(const Bodies& B, int j,
 // the records do not reach tn. The bracketing records are kept in the
 // body's segment cache and refilled from its contiguous (CSR) records when
 // tn leaves the segment. L holds the body's preloaded inputs.
+template <bool kRound>
 __device__ __forceinline__ void predict_body(const Bodies& B, const Params& P,
                                              const History& prev, int j,
                                              int slot, long long tj,
@@ -201,7 +210,7 @@ __device__ __forceinline__ void predict_body(const Bodies& B, const Params& P,
       }
     }
   }
-  store_prediction(B, P, j, slot, rp, vp);
+  store_prediction<kRound>(B, P, j, slot, rp, vp);
 }
 
 // S split partial sums of active position k (layout [split][5][n_act]),

@@ -8,6 +8,12 @@ errors leave (five standard deviations of 0.29 units / sqrt(count)), with x's
 upper part cut toward zero as the integrator cuts it, and rounded as the force
 call does.
 
+The split of a coordinate in ordered runs has its upper part rounded to nearest
+and is exact to 2^-49. With it the distances of both forms of a pair, the
+double-single difference and the one about a centre, have the same mean: none
+beyond 5e-10 of the distance, where 300,000 pairs leave 1.2e-10 of their 3e-8
+each (four standard deviations, both forms; cut upper parts leave 3e-9).
+
 The curve's cells are the bodies' own: a Plummer sphere that was moved has as
 many far pairs of a warp's bodies and a subtile as one about the coordinate
 origin (within a tenth; the cells' edges lie elsewhere), also with a body far
@@ -30,6 +36,9 @@ WRAP = r"""
 extern "C" void about_n(long long n, const float* h, const float* l, float c,
                         float* out) {
   for (long long i = 0; i < n; ++i) out[i] = tsbts::about(h[i], l[i], c);
+}
+extern "C" void split_n(long long n, const double* x, float* h, float* l) {
+  for (long long i = 0; i < n; ++i) tsbts::split_round(x[i], h[i], l[i]);
 }
 extern "C" void sample_n(int n, int* out) {
   for (int k = 0; k < tsbts::kCentreSample; ++k)
@@ -59,6 +68,7 @@ def lib(tmp_path_factory):
                     str(src), "-o", str(so)], check=True)
     L = C.CDLL(str(so))
     L.about_n.argtypes = [C.c_longlong, FP, FP, C.c_float, FP]
+    L.split_n.argtypes = [C.c_longlong, C.POINTER(C.c_double), FP, FP]
     L.sample_n.argtypes = [C.c_int, C.POINTER(C.c_int)]
     L.keys_n.argtypes = [C.c_longlong, FP, C.c_float, C.POINTER(C.c_uint32)]
     return L
@@ -95,6 +105,52 @@ def test_one_rounding(lib, cut, c, shift):
             2.0 ** -48 * np.abs(x)).all()
     toward = (err / unit) * np.sign(x)
     assert abs(toward.mean()) < 5 * 0.29 / np.sqrt(len(x))
+
+
+def _split_round(lib, x):
+    x = np.ascontiguousarray(x)
+    h, l = np.empty(x.shape, np.float32), np.empty(x.shape, np.float32)
+    lib.split_n(x.size, x.ctypes.data_as(C.POINTER(C.c_double)),
+                h.ctypes.data_as(FP), l.ctypes.data_as(FP))
+    return h, l
+
+
+def test_split_rounds_to_nearest(lib):
+    g = np.random.default_rng(4)
+    x = g.choice([-1.0, 1.0], 200000) * 2.0 ** g.uniform(-70, 100, 200000)
+    x[:4] = [1.0, -1.0, 1.0 + 2.0 ** -24, np.nextafter(2.0, 0.0)]
+    h, l = _split_round(lib, x)
+    unit = np.spacing(np.abs(x).astype(np.float32)).astype(np.float64)
+    assert (np.abs(h - x) <= 0.5 * unit).all()
+    assert (np.abs(h.astype(np.float64) + l - x) <=
+            2.0 ** -49 * np.abs(x)).all()
+    assert (h[4:] == x[4:].astype(np.float32)).all()
+
+
+def test_both_forms_of_a_pair_have_the_same_mean(lib):
+    r = inputs.plummer(36864, 1)[1]
+    h, l = _split_round(lib, r)
+    g = np.random.default_rng(0)
+    err = {"near": [], "far": []}
+    while len(err["far"]) < 75:
+        d2 = ((r - r[g.integers(len(r))]) ** 2).sum(1)
+        block = np.argsort(d2)[:256]
+        lo, hi = h[block].min(0), h[block].max(0)
+        cen = np.float32(0.5) * (lo + hi)
+        rho2 = ((hi - lo).astype(np.float64) ** 2).sum() / 4
+        j = np.flatnonzero(d2 > 6.25 * rho2)
+        if len(j) < 1000:
+            continue
+        j, i = g.choice(j, 4000), g.choice(block, 4000)
+        d = r[j] - r[i]
+        far = np.stack([_about(lib, np.ascontiguousarray(h[:, k]),
+                               np.ascontiguousarray(l[:, k]), cen[k])
+                        for k in range(3)], 1)
+        for name, x in (("near", (h[j] - h[i]) + (l[j] - l[i])),
+                        ("far", far[j] - far[i])):
+            err[name].append((((x - d) * d).sum(1) / (d * d).sum(1)).mean())
+    for name, e in err.items():
+        assert abs(np.mean(e)) < 5e-10, (name, np.mean(e))
 
 
 def spatial_order(lib, r):
