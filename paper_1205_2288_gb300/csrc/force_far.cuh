@@ -5,12 +5,14 @@
 // small boxes. Most pairs of a warp and a subtile are then far apart, and
 // far pairs need less work for the same result:
 //  - coordinates: x'_j = x_j - c and x'_i = x_i - c, each rounded once to
-//    FP32 about the centre c of the block's 256 bodies (far_rule.h: once per
-//    staged j, 3 of 250 additions a pair), leave one subtraction per
-//    component instead of the three of the double-single difference. Where the boxes are further apart than the radius rho of
-//    those bodies, |x'_j| + |x'_i| <= 3 |d|, so the rounding of x'_j and
-//    x'_i is at most 3/2 units of d's last place, as the two roundings of the
-//    double-single difference of far bodies are one;
+//    FP32 about the centre c of the block's 256 bodies (far_rule.h; once per
+//    staged j), leave one subtraction per component instead of the three of
+//    the double-single difference. Where the boxes are further apart than the
+//    radius rho of those bodies, |x'_j| + |x'_i| <= 3 |d|, so the rounding of
+//    x'_j and x'_i is at most 3/2 units of d's last place, as the two
+//    roundings of the double-single difference of far bodies are one. Neither
+//    form's distances have a mean error (split_round): one that differs
+//    between them would change a pair's force when it crosses over;
 //  - the step criterion: q_i is a maximum, so a subtile whose largest possible
 //    term, max((v_i + v_j)^2 / s^2, m_j / s^3) at the boxes' distance with the
 //    largest speeds and mass in them, is below the q that every body of the
@@ -20,7 +22,7 @@
 // A far pair then takes 13 FMA-pipe operations and about 31 register reads
 // instead of 26 and 57, a near one without the criterion 19 and 41. Of the
 // pairs of all of 131072 bodies three quarters are far, of 16384 a quarter.
-// All of 131072 bodies: 11.3 ms with both sorts, 14.65 in the unsorted form;
+// All of 131072 bodies: 11.4 ms with both sorts, 14.65 in the unsorted form;
 // the start of their era 269 ms, 389 before. Errors against 64 bits (relative
 // 2-norms): a 2.7e-8 (3.2e-8 unsorted), phi 7e-9 (9e-9), q 1.1e-7 (1.1e-7).
 #pragma once
